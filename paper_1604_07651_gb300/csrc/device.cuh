@@ -1,0 +1,102 @@
+// Device and launch helpers shared by the kernel files: the piece of a block
+// in a batched launch, shared-memory checks and limits.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <mutex>
+#include <vector>
+
+#include "internal.h"
+
+namespace hr {
+
+extern __shared__ __align__(16) float smem_f[];
+
+// Piece of this block in a batched launch, and the block's index within it:
+// from the descriptors passed as a kernel parameter (up to kMaxBatch pieces)
+// or from a device-resident batch (any number of pieces of many gathers).
+__device__ __forceinline__ int batch_piece(const PieceBatch& B, int& bx) {
+    int pi = 0;
+#pragma unroll
+    for (int k = 1; k < kMaxBatch; ++k)
+        if (k < B.n && (int)blockIdx.x >= B.first[k]) pi = k;
+    bx = (int)blockIdx.x - B.first[pi];
+    return pi;
+}
+__device__ __forceinline__ const PieceDev& piece_of(const PieceBatch& B, int& bx) { return B.p[batch_piece(B, bx)]; }
+__device__ __forceinline__ const PieceDev& piece_of(const DevBatch& B, int& bx) {
+    const int2 m = __ldg(B.map + blockIdx.x);
+    bx = m.y;
+    return B.p[m.x];
+}
+
+// The radices of pass 0 (dif_plan).
+#define HR_RADIX_CASES(CALL) \
+    case 16: CALL(16); break; \
+    case 12: CALL(12); break; \
+    case 10: CALL(10); break; \
+    case 9: CALL(9); break;   \
+    case 8: CALL(8); break;   \
+    case 6: CALL(6); break;   \
+    case 5: CALL(5); break;   \
+    case 4: CALL(4); break;   \
+    case 3: CALL(3); break;   \
+    default: CALL(2); break;
+
+// Dynamic shared memory of the launch: the row and column kernels check it
+// against what their piece needs and leave the block untouched (never write
+// past it) if a launch gave too little.
+__device__ __forceinline__ unsigned dyn_smem_bytes() {
+    unsigned r;
+    asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(r));
+    return r;
+}
+
+inline int check_launch() {
+    cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? 0 : (int)e;
+}
+
+// Dynamic shared-memory limit of a kernel: raised only when a launch needs
+// more than the largest value already set on this device (the attribute call
+// costs host time on every launch otherwise).
+inline int set_smem(const void* fn, size_t bytes) {
+    struct Entry { const void* fn; int dev; size_t bytes; };
+    static std::mutex mu;
+    static std::vector<Entry> set;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lock(mu);
+    for (const Entry& e : set)
+        if (e.fn == fn && e.dev == dev && e.bytes >= bytes) return 0;
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e != cudaSuccess) return (int)e;
+    for (Entry& en : set)
+        if (en.fn == fn && en.dev == dev) {
+            en.bytes = bytes;
+            return 0;
+        }
+    set.push_back(Entry{fn, dev, bytes});
+    return 0;
+}
+
+// Batch descriptor of n pieces with count(piece) blocks each; returns the
+// total number of blocks.
+template <class F>
+inline int make_batch(const PieceDev* P, int n, PieceBatch& B, F&& count) {
+    B.n = n;
+    int total = 0;
+    for (int k = 0; k < kMaxBatch; ++k) {
+        B.first[k] = total;
+        if (k < n) {
+            B.p[k] = P[k];
+            total += count(P[k]);
+        }
+    }
+    B.first[kMaxBatch] = total;
+    return total;
+}
+
+}  // namespace hr

@@ -71,41 +71,111 @@ HD cf cmulc(cf a, cf b) { return {a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y};
 HD cf cadd(cf a, cf b) { return {a.x + b.x, a.y + b.y}; }
 HD cf csub(cf a, cf b) { return {a.x - b.x, a.y - b.y}; }
 HD cf cconj(cf a) { return {a.x, -a.y}; }
+// The operations of the in-register DFTs, on one complex number (cf) here and
+// on the same element of two sequences at once in the kernels (fft2.cuh):
+// a + i b, a - i b, the product with a constant, a + s b and s a for real s.
+HD cf caddi(cf a, cf b) { return {a.x - b.y, a.y + b.x}; }
+HD cf csubi(cf a, cf b) { return {a.x + b.y, a.y - b.x}; }
+HD cf cmulk(cf a, float re, float im) { return {a.x * re - a.y * im, a.x * im + a.y * re}; }
+HD cf caxpy(cf a, float s, cf b) { return {a.x + s * b.x, a.y + s * b.y}; }
+HD cf cscale(float s, cf a) { return {s * a.x, s * a.y}; }
 
-// In-register DFT of size R (2, 3 or 4) with sign dir (-1 forward, +1 inverse).
+// In-register DFT of size R (2, 3, 4, 5, 6, 8, 9, 10, 12, 16) with sign dir
+// (-1 forward, +1 inverse; a compile-time constant after inlining), for any
+// element type with the operations above.
 template <int R>
-HD void dft_small(cf v[R], int dir);
+struct Dft;
+template <int R, class C>
+HD void dft_small(C* v, int dir) { Dft<R>::template run<R>(v, dir); }
+// The same when the inputs from NZ on are zero (they are not read): the
+// zero-padded half of an FFT's first pass.
+template <int R, int NZ, class C>
+HD void dft_zeros(C* v, int dir) { Dft<R>::template run<NZ>(v, dir); }
+template <int R, int NZ, class C>
+HD void dft_lead(C* v, int dir);
+// Inputs below NZ among the every-F-th ones n2, n2 + F, ... of a size-R DFT.
+HD constexpr int lead_count(int NZ, int F, int n2) { return NZ > n2 ? (NZ - n2 + F - 1) / F : 0; }
 
 template <>
-HD void dft_small<2>(cf v[2], int) {
-    cf a = v[0], b = v[1];
-    v[0] = cadd(a, b);
-    v[1] = csub(a, b);
-}
+struct Dft<2> {
+    template <int NZ, class C>
+    HD static void run(C* v, int) {
+        if (NZ == 1) {
+            v[1] = v[0];
+            return;
+        }
+        const C a = v[0], b = v[1];
+        v[0] = cadd(a, b);
+        v[1] = csub(a, b);
+    }
+};
 
 template <>
-HD void dft_small<4>(cf v[4], int dir) {
-    cf a0 = cadd(v[0], v[2]), a1 = csub(v[0], v[2]);
-    cf b0 = cadd(v[1], v[3]), b1 = csub(v[1], v[3]);
-    // b1 * (dir * i)
-    cf jb1 = dir < 0 ? cf{b1.y, -b1.x} : cf{-b1.y, b1.x};
-    v[0] = cadd(a0, b0);
-    v[2] = csub(a0, b0);
-    v[1] = cadd(a1, jb1);
-    v[3] = csub(a1, jb1);
-}
+struct Dft<4> {
+    template <int NZ, class C>
+    HD static void run(C* v, int dir) {
+        if (NZ < 3) return dft_lead<4, NZ>(v, dir);
+        const C a0 = cadd(v[0], v[2]), a1 = csub(v[0], v[2]);
+        const C b0 = cadd(v[1], v[3]), b1 = csub(v[1], v[3]);
+        v[0] = cadd(a0, b0);
+        v[2] = csub(a0, b0);
+        v[1] = dir < 0 ? csubi(a1, b1) : caddi(a1, b1);
+        v[3] = dir < 0 ? caddi(a1, b1) : csubi(a1, b1);
+    }
+};
 
 template <>
-HD void dft_small<3>(cf v[3], int dir) {
-    const float c = -0.5f;
-    const float s = 0.86602540378443864676f * (float)dir;  // sin(2 pi/3) * dir
-    cf t = cadd(v[1], v[2]);
-    cf d = csub(v[1], v[2]);
-    cf m = {v[0].x + c * t.x, v[0].y + c * t.y};
-    cf id = {-s * d.y, s * d.x};  // i * s * d
-    v[0] = cadd(v[0], t);
-    v[1] = cadd(m, id);
-    v[2] = csub(m, id);
+struct Dft<3> {
+    template <int NZ, class C>
+    HD static void run(C* v, int dir) {
+        if (NZ < 3) return dft_lead<3, NZ>(v, dir);
+        const float s = 0.86602540378443864676f * (float)dir;  // sin(2 pi/3) * dir
+        const C t = cadd(v[1], v[2]);
+        const C d = cscale(s, csub(v[1], v[2]));
+        const C m = caxpy(v[0], -0.5f, t);
+        v[0] = cadd(v[0], t);
+        v[1] = caddi(m, d);
+        v[2] = csubi(m, d);
+    }
+};
+
+// DFTs of size 3, 4 and 5 whose inputs from NZ on are zero.
+template <int R, int NZ, class C>
+HD void dft_lead(C* v, int dir) {
+    if (NZ >= R || (R == 4 && NZ == 3) || (R == 5 && NZ == 4)) {
+        dft_small<R>(v, dir);
+    } else if (NZ == 1) {
+HD_UNROLL
+        for (int k = 1; k < R; ++k) v[k] = v[0];
+    } else if (R == 3) {                                   // two inputs
+        const C m = caxpy(v[0], -0.5f, v[1]), d = cscale(0.86602540378443864676f * (float)dir, v[1]);
+        v[0] = cadd(v[0], v[1]);
+        v[1] = caddi(m, d);
+        v[2] = csubi(m, d);
+    } else if (R == 4) {
+        const C a = v[0], b = v[1];
+        v[0] = cadd(a, b);
+        v[2] = csub(a, b);
+        v[1] = dir < 0 ? csubi(a, b) : caddi(a, b);
+        v[3] = dir < 0 ? caddi(a, b) : csubi(a, b);
+    } else {                                               // R == 5, two or three inputs
+        const float c1 = 0.30901699437494742410f, c2 = -0.80901699437494742410f;
+        const float s1 = 0.95105651629515357212f * (float)dir, s2 = 0.58778525229247312917f * (float)dir;
+        C a1 = caxpy(v[0], c1, v[1]), a2 = caxpy(v[0], c2, v[1]), b1 = cscale(s1, v[1]), b2 = cscale(s2, v[1]);
+        C sum = cadd(v[0], v[1]);
+        if (NZ == 3) {
+            a1 = caxpy(a1, c2, v[2]);
+            a2 = caxpy(a2, c1, v[2]);
+            b1 = caxpy(b1, s2, v[2]);
+            b2 = caxpy(b2, -s1, v[2]);
+            sum = cadd(sum, v[2]);
+        }
+        v[0] = sum;
+        v[1] = caddi(a1, b1);
+        v[4] = csubi(a1, b1);
+        v[2] = caddi(a2, b2);
+        v[3] = csubi(a2, b2);
+    }
 }
 
 // cos(2 pi i / 16); with i a compile-time constant after unrolling, the
@@ -123,16 +193,7 @@ HD float cos16(int i) {
         default: return -1.0f;
     }
 }
-
-// exp(dir * 2 pi i k / N) for the in-register DFTs of size 8 and 16.
-template <int N>
-HD cf unit_root(int k, int dir) {
-    const int i = k * (16 / N);
-    return {cos16(i), dir * cos16(i - 4)};   // sin(x) = cos(x - pi/2)
-}
-
-// exp(dir * 2 pi i m / 12) for the in-register DFTs of size 6 and 12; m is
-// a compile-time constant after unrolling.
+// cos(2 pi m / 12) and cos(2 pi m / 10), as above.
 HD float cos12(int i) {
     switch (((i % 12) + 12) % 12) {
         case 0: return 1.0f;
@@ -144,94 +205,6 @@ HD float cos12(int i) {
         default: return -1.0f;
     }
 }
-HD cf root12(int m, int dir) { return {cos12(m), dir * cos12(m - 3)}; }
-
-// Size 6 as 3 x 2 and size 12 as 3 x 4 (Cooley-Tukey with n = F n1 + n2,
-// k = k1 + 3 k2): Y[n2][k1] = DFT3 over n1 of x[F n1 + n2], times
-// W^(n2 k1), then X[k1 + 3 k2] = DFT-F over n2.
-template <int F>
-HD void dft_3xF(cf v[3 * F], int dir) {
-    cf y[F][3];
-HD_UNROLL
-    for (int n2 = 0; n2 < F; ++n2) {
-HD_UNROLL
-        for (int n1 = 0; n1 < 3; ++n1) y[n2][n1] = v[F * n1 + n2];
-        dft_small<3>(y[n2], dir);
-    }
-HD_UNROLL
-    for (int k1 = 0; k1 < 3; ++k1) {
-        cf z[F];
-HD_UNROLL
-        for (int n2 = 0; n2 < F; ++n2)
-            z[n2] = (n2 * k1 != 0) ? cmul(y[n2][k1], root12(n2 * k1 * (12 / (3 * F)), dir)) : y[n2][k1];
-        dft_small<F>(z, dir);
-HD_UNROLL
-        for (int k2 = 0; k2 < F; ++k2) v[k1 + 3 * k2] = z[k2];
-    }
-}
-
-template <>
-HD void dft_small<6>(cf v[6], int dir) { dft_3xF<2>(v, dir); }
-
-template <>
-HD void dft_small<12>(cf v[12], int dir) { dft_3xF<4>(v, dir); }
-
-// exp(dir * 2 pi i m / 9) for m = 1, 2, 4, the twiddles of the 3 x 3 split
-// (cos and sin of 40, 80 and 160 degrees).
-HD cf root9(int m, int dir) {
-    switch (m) {
-        case 1: return {0.76604444311897803520f, dir * 0.64278760968653932632f};
-        case 2: return {0.17364817766693034885f, dir * 0.98480775301220805936f};
-        default: return {-0.93969262078590838405f, dir * 0.34202014332566873304f};
-    }
-}
-
-// Size 9 as 3 x 3 (Cooley-Tukey with n = 3 n1 + n2, k = k1 + 3 k2):
-// Y[n2][k1] = DFT3 over n1 of x[3 n1 + n2], times W9^(n2 k1), then
-// X[k1 + 3 k2] = DFT3 over n2.
-template <>
-HD void dft_small<9>(cf v[9], int dir) {
-    cf y[3][3];
-HD_UNROLL
-    for (int n2 = 0; n2 < 3; ++n2) {
-HD_UNROLL
-        for (int n1 = 0; n1 < 3; ++n1) y[n2][n1] = v[3 * n1 + n2];
-        dft_small<3>(y[n2], dir);
-    }
-HD_UNROLL
-    for (int k1 = 0; k1 < 3; ++k1) {
-        cf z[3];
-HD_UNROLL
-        for (int n2 = 0; n2 < 3; ++n2) z[n2] = (n2 * k1 != 0) ? cmul(y[n2][k1], root9(n2 * k1, dir)) : y[n2][k1];
-        dft_small<3>(z, dir);
-HD_UNROLL
-        for (int k2 = 0; k2 < 3; ++k2) v[k1 + 3 * k2] = z[k2];
-    }
-}
-
-// Size 5 directly: with t1 = x1 + x4, t2 = x2 + x3, t3 = x1 - x4,
-// t4 = x2 - x3 and c_m = cos(2 pi m / 5), s_m = sin(2 pi m / 5):
-// X1,4 = x0 + c1 t1 + c2 t2 +- i dir (s1 t3 + s2 t4),
-// X2,3 = x0 + c2 t1 + c1 t2 +- i dir (s2 t3 - s1 t4).
-template <>
-HD void dft_small<5>(cf v[5], int dir) {
-    const float c1 = 0.30901699437494742410f, c2 = -0.80901699437494742410f;   // (sqrt5 - 1)/4, -(sqrt5 + 1)/4
-    const float s1 = 0.95105651629515357212f * (float)dir, s2 = 0.58778525229247312917f * (float)dir;
-    const cf t1 = cadd(v[1], v[4]), t2 = cadd(v[2], v[3]);
-    const cf t3 = csub(v[1], v[4]), t4 = csub(v[2], v[3]);
-    const cf a1 = {v[0].x + c1 * t1.x + c2 * t2.x, v[0].y + c1 * t1.y + c2 * t2.y};
-    const cf a2 = {v[0].x + c2 * t1.x + c1 * t2.x, v[0].y + c2 * t1.y + c1 * t2.y};
-    const cf b1 = {s1 * t3.x + s2 * t4.x, s1 * t3.y + s2 * t4.y};
-    const cf b2 = {s2 * t3.x - s1 * t4.x, s2 * t3.y - s1 * t4.y};
-    v[0] = cadd(v[0], cadd(t1, t2));
-    v[1] = {a1.x - b1.y, a1.y + b1.x};   // a1 + i b1
-    v[4] = {a1.x + b1.y, a1.y - b1.x};   // a1 - i b1
-    v[2] = {a2.x - b2.y, a2.y + b2.x};
-    v[3] = {a2.x + b2.y, a2.y - b2.x};
-}
-
-// cos(2 pi m / 10) and exp(dir * 2 pi i m / 10), m a compile-time constant
-// after unrolling.
 HD float cos10(int i) {
     switch (((i % 10) + 10) % 10) {
         case 0: return 1.0f;
@@ -252,61 +225,212 @@ HD float sin10(int i) {
     }
 }
 
+// v times exp(dir * 2 pi i m / 16) or / 12; a quarter turn (m = N / 4) is a
+// swap done by the caller's caddi / csubi where it can be, here by a product
+// with (0, dir).
+template <class C>
+HD C turn16(C v, int m, int dir) { return m ? cmulk(v, cos16(m), dir * cos16(m - 4)) : v; }   // sin(x) = cos(x - pi/2)
+template <class C>
+HD C turn12(C v, int m, int dir) { return m ? cmulk(v, cos12(m), dir * cos12(m - 3)) : v; }
+
+// Size 6 as 3 x 2 and size 12 as 3 x 4 (Cooley-Tukey with n = F n1 + n2,
+// k = k1 + 3 k2): Y[n2][k1] = DFT3 over n1 of x[F n1 + n2], times
+// W^(n2 k1), then X[k1 + 3 k2] = DFT-F over n2.
+template <int F, int NZ, class C>
+HD void dft_3xF(C* v, int dir) {
+    C y[F][3];
+HD_UNROLL
+    for (int n2 = 0; n2 < F; ++n2) {
+HD_UNROLL
+        for (int n1 = 0; n1 < 3; ++n1)
+            if (F * n1 + n2 < NZ) y[n2][n1] = v[F * n1 + n2];
+    }
+    dft_lead<3, lead_count(NZ, F, 0)>(y[0], dir);
+    dft_lead<3, lead_count(NZ, F, 1)>(y[1], dir);
+    if (F > 2) {
+        dft_lead<3, lead_count(NZ, F, 2)>(y[F > 2 ? 2 : 0], dir);
+        dft_lead<3, lead_count(NZ, F, 3)>(y[F > 2 ? 3 : 0], dir);
+    }
+HD_UNROLL
+    for (int k1 = 0; k1 < 3; ++k1) {
+        C z[F];
+HD_UNROLL
+        for (int n2 = 0; n2 < F; ++n2) z[n2] = turn12(y[n2][k1], n2 * k1 * (12 / (3 * F)), dir);
+        dft_small<F>(z, dir);
+HD_UNROLL
+        for (int k2 = 0; k2 < F; ++k2) v[k1 + 3 * k2] = z[k2];
+    }
+}
+
+template <>
+struct Dft<6> {
+    template <int NZ, class C>
+    HD static void run(C* v, int dir) { dft_3xF<2, NZ>(v, dir); }
+};
+
+template <>
+struct Dft<12> {
+    template <int NZ, class C>
+    HD static void run(C* v, int dir) { dft_3xF<4, NZ>(v, dir); }
+};
+
+// exp(dir * 2 pi i m / 9) for m = 1, 2, 4, the twiddles of the 3 x 3 split
+// (cos and sin of 40, 80 and 160 degrees).
+HD cf root9(int m, int dir) {
+    switch (m) {
+        case 1: return {0.76604444311897803520f, dir * 0.64278760968653932632f};
+        case 2: return {0.17364817766693034885f, dir * 0.98480775301220805936f};
+        default: return {-0.93969262078590838405f, dir * 0.34202014332566873304f};
+    }
+}
+
+// Size 9 as 3 x 3 (Cooley-Tukey with n = 3 n1 + n2, k = k1 + 3 k2):
+// Y[n2][k1] = DFT3 over n1 of x[3 n1 + n2], times W9^(n2 k1), then
+// X[k1 + 3 k2] = DFT3 over n2.
+template <>
+struct Dft<9> {
+    template <int NZ, class C>
+    HD static void run(C* v, int dir) {
+        C y[3][3];
+HD_UNROLL
+        for (int n2 = 0; n2 < 3; ++n2) {
+HD_UNROLL
+            for (int n1 = 0; n1 < 3; ++n1)
+                if (3 * n1 + n2 < NZ) y[n2][n1] = v[3 * n1 + n2];
+        }
+        dft_lead<3, lead_count(NZ, 3, 0)>(y[0], dir);
+        dft_lead<3, lead_count(NZ, 3, 1)>(y[1], dir);
+        dft_lead<3, lead_count(NZ, 3, 2)>(y[2], dir);
+HD_UNROLL
+        for (int k1 = 0; k1 < 3; ++k1) {
+            C z[3];
+HD_UNROLL
+            for (int n2 = 0; n2 < 3; ++n2)
+                z[n2] = (n2 * k1 != 0) ? cmulk(y[n2][k1], root9(n2 * k1, dir).x, root9(n2 * k1, dir).y) : y[n2][k1];
+            dft_small<3>(z, dir);
+HD_UNROLL
+            for (int k2 = 0; k2 < 3; ++k2) v[k1 + 3 * k2] = z[k2];
+        }
+    }
+};
+
+// Size 5 directly: with t1 = x1 + x4, t2 = x2 + x3, t3 = x1 - x4,
+// t4 = x2 - x3 and c_m = cos(2 pi m / 5), s_m = sin(2 pi m / 5):
+// X1,4 = x0 + c1 t1 + c2 t2 +- i dir (s1 t3 + s2 t4),
+// X2,3 = x0 + c2 t1 + c1 t2 +- i dir (s2 t3 - s1 t4).
+template <>
+struct Dft<5> {
+    template <int NZ, class C>
+    HD static void run(C* v, int dir) {
+        if (NZ < 4) return dft_lead<5, NZ>(v, dir);
+        const float c1 = 0.30901699437494742410f, c2 = -0.80901699437494742410f;   // (sqrt5 - 1)/4, -(sqrt5 + 1)/4
+        const float s1 = 0.95105651629515357212f * (float)dir, s2 = 0.58778525229247312917f * (float)dir;
+        const C t1 = cadd(v[1], v[4]), t2 = cadd(v[2], v[3]);
+        const C t3 = csub(v[1], v[4]), t4 = csub(v[2], v[3]);
+        const C a1 = caxpy(caxpy(v[0], c1, t1), c2, t2);
+        const C a2 = caxpy(caxpy(v[0], c2, t1), c1, t2);
+        const C b1 = caxpy(cscale(s1, t3), s2, t4);
+        const C b2 = caxpy(cscale(s2, t3), -s1, t4);
+        v[0] = cadd(v[0], cadd(t1, t2));
+        v[1] = caddi(a1, b1);
+        v[4] = csubi(a1, b1);
+        v[2] = caddi(a2, b2);
+        v[3] = csubi(a2, b2);
+    }
+};
+
 // Size 10 as 5 x 2: Y[n2][k1] = DFT5 over n1 of x[2 n1 + n2], times
 // W10^(n2 k1), then X[k1 + 5 k2] = DFT2 over n2.
 template <>
-HD void dft_small<10>(cf v[10], int dir) {
-    cf y0[5], y1[5];
+struct Dft<10> {
+    template <int NZ, class C>
+    HD static void run(C* v, int dir) {
+        C y0[5], y1[5];
 HD_UNROLL
-    for (int n1 = 0; n1 < 5; ++n1) {
-        y0[n1] = v[2 * n1];
-        y1[n1] = v[2 * n1 + 1];
-    }
-    dft_small<5>(y0, dir);
-    dft_small<5>(y1, dir);
+        for (int n1 = 0; n1 < 5; ++n1) {
+            if (2 * n1 < NZ) y0[n1] = v[2 * n1];
+            if (2 * n1 + 1 < NZ) y1[n1] = v[2 * n1 + 1];
+        }
+        dft_lead<5, lead_count(NZ, 2, 0)>(y0, dir);
+        dft_lead<5, lead_count(NZ, 2, 1)>(y1, dir);
 HD_UNROLL
-    for (int k1 = 0; k1 < 5; ++k1) {
-        const cf t = k1 ? cmul(y1[k1], cf{cos10(k1), dir * sin10(k1)}) : y1[k1];
-        v[k1] = cadd(y0[k1], t);
-        v[k1 + 5] = csub(y0[k1], t);
+        for (int k1 = 0; k1 < 5; ++k1) {
+            const C t = k1 ? cmulk(y1[k1], cos10(k1), dir * sin10(k1)) : y1[k1];
+            v[k1] = cadd(y0[k1], t);
+            v[k1 + 5] = csub(y0[k1], t);
+        }
     }
-}
+};
 
-// Size 8 as 2 x 4: inputs x[2 n1 + n2], X[k1 + 4 k2].
+// Size 8 as 2 x 4: inputs x[2 n1 + n2], X[k1 + 4 k2]; the quarter turn of
+// k1 = 2 is folded into the last butterfly.
 template <>
-HD void dft_small<8>(cf v[8], int dir) {
-    cf e[4] = {v[0], v[2], v[4], v[6]}, o[4] = {v[1], v[3], v[5], v[7]};
-    dft_small<4>(e, dir);
-    dft_small<4>(o, dir);
+struct Dft<8> {
+    template <int NZ, class C>
+    HD static void run(C* v, int dir) {
+        C e[4], o[4];
 HD_UNROLL
-    for (int k = 0; k < 4; ++k) {
-        const cf t = k ? cmul(o[k], unit_root<8>(k, dir)) : o[k];
-        v[k] = cadd(e[k], t);
-        v[k + 4] = csub(e[k], t);
+        for (int n1 = 0; n1 < 4; ++n1) {
+            if (2 * n1 < NZ) e[n1] = v[2 * n1];
+            if (2 * n1 + 1 < NZ) o[n1] = v[2 * n1 + 1];
+        }
+        dft_lead<4, lead_count(NZ, 2, 0)>(e, dir);
+        dft_lead<4, lead_count(NZ, 2, 1)>(o, dir);
+HD_UNROLL
+        for (int k = 0; k < 4; ++k) {
+            if (k == 2) {
+                v[k] = dir < 0 ? csubi(e[k], o[k]) : caddi(e[k], o[k]);
+                v[k + 4] = dir < 0 ? caddi(e[k], o[k]) : csubi(e[k], o[k]);
+            } else {
+                const C t = turn16(o[k], 2 * k, dir);
+                v[k] = cadd(e[k], t);
+                v[k + 4] = csub(e[k], t);
+            }
+        }
     }
-}
+};
 
 // Size 16 as 4 x 4: Y[n2][k1] = DFT4 over n1 of x[4 n1 + n2], times
-// W16^(n2 k1), then X[k1 + 4 k2] = DFT4 over n2.
+// W16^(n2 k1), then X[k1 + 4 k2] = DFT4 over n2; the quarter turn of
+// n2 k1 = 4 (n2 = k1 = 2) is folded into that DFT4's first butterfly.
 template <>
-HD void dft_small<16>(cf v[16], int dir) {
-    cf y[4][4];
+struct Dft<16> {
+    template <int NZ, class C>
+    HD static void run(C* v, int dir) {
+        C y[4][4];
 HD_UNROLL
-    for (int n2 = 0; n2 < 4; ++n2) {
+        for (int n2 = 0; n2 < 4; ++n2) {
 HD_UNROLL
-        for (int n1 = 0; n1 < 4; ++n1) y[n2][n1] = v[4 * n1 + n2];
-        dft_small<4>(y[n2], dir);
+            for (int n1 = 0; n1 < 4; ++n1)
+                if (4 * n1 + n2 < NZ) y[n2][n1] = v[4 * n1 + n2];
+        }
+        dft_lead<4, lead_count(NZ, 4, 0)>(y[0], dir);
+        dft_lead<4, lead_count(NZ, 4, 1)>(y[1], dir);
+        dft_lead<4, lead_count(NZ, 4, 2)>(y[2], dir);
+        dft_lead<4, lead_count(NZ, 4, 3)>(y[3], dir);
+HD_UNROLL
+        for (int k1 = 0; k1 < 4; ++k1) {
+            C z[4];
+HD_UNROLL
+            for (int n2 = 0; n2 < 4; ++n2)
+                z[n2] = n2 * k1 == 4 ? y[n2][k1] : turn16(y[n2][k1], n2 * k1, dir);
+            if (k1 == 2) {
+                const bool plus = dir > 0;
+                const C a0 = plus ? caddi(z[0], z[2]) : csubi(z[0], z[2]);
+                const C a1 = plus ? csubi(z[0], z[2]) : caddi(z[0], z[2]);
+                const C b0 = cadd(z[1], z[3]), b1 = csub(z[1], z[3]);
+                z[0] = cadd(a0, b0);
+                z[2] = csub(a0, b0);
+                z[1] = plus ? caddi(a1, b1) : csubi(a1, b1);
+                z[3] = plus ? csubi(a1, b1) : caddi(a1, b1);
+            } else {
+                dft_small<4>(z, dir);
+            }
+HD_UNROLL
+            for (int k2 = 0; k2 < 4; ++k2) v[k1 + 4 * k2] = z[k2];
+        }
     }
-HD_UNROLL
-    for (int k1 = 0; k1 < 4; ++k1) {
-        cf z[4];
-HD_UNROLL
-        for (int n2 = 0; n2 < 4; ++n2) z[n2] = (n2 * k1 != 0) ? cmul(y[n2][k1], unit_root<16>(n2 * k1, dir)) : y[n2][k1];
-        dft_small<4>(z, dir);
-HD_UNROLL
-        for (int k2 = 0; k2 < 4; ++k2) v[k1 + 4 * k2] = z[k2];
-    }
-}
+};
 
 // Twiddle table of one FFT pass with Ns butterflies per block and radix R:
 // entry (r - 1) Ns + jm is exp(-2 pi i r jm / (Ns R)), r = 1 .. R-1,
@@ -462,24 +586,25 @@ inline int fft_dif_tables(int n, cf* T) {
 // are zero for a real signal), Z[0] = X0 + i X0.
 HD cf c2r_pre_dc(cf X0) { return {X0.x, X0.x}; }
 
-// The row kernels hold Z in digit-reversed order: the forward step reads
-// Z[k] and Z[M-k] from buffer positions pk and pmk;
-HD cf r2c_post_at(const cf* Z, int pk, int pmk, int k, const cf* twP) {
-    cf a = Z[pk];
-    cf b = cconj(Z[pmk]);
-    cf e = cadd(a, b);
-    cf o = cmul(twP[k], csub(a, b));
-    return {e.x + o.y, e.y - o.x};
-}
+// a + conj(b), a - conj(b) and conj(a - i b).
+HD cf cadd_conj(cf a, cf b) { return {a.x + b.x, a.y - b.y}; }
+HD cf csub_conj(cf a, cf b) { return {a.x - b.x, a.y + b.y}; }
+HD cf conj_subi(cf a, cf b) { return {a.x + b.y, b.x - a.y}; }
+
+// The forward step from Zk = Z[k], Zmk = Z[M-k] and w = W^k, for any element
+// type with these operations (two rows at once in the kernels);
+template <class C>
+HD C r2c_post(C Zk, C Zmk, C w) { return csubi(cadd_conj(Zk, Zmk), cmul(csub_conj(Zk, Zmk), w)); }
+// with Z in digit-reversed order, read at positions pk and pmk;
+HD cf r2c_post_at(const cf* Z, int pk, int pmk, int k, const cf* twP) { return r2c_post(Z[pk], Z[pmk], twP[k]); }
 // the inverse step takes a = X[k], b = X[M-k] and w = W^k and gives the
-// packed inputs Z[k] (zk) and Z[M-k] (zmk), 0 < k < M.
-HD void c2r_pre_vals(cf a, cf b, cf w, cf& zk, cf& zmk) {
-    cf e1 = cadd(a, cconj(b));
-    cf o1 = cmulc(csub(a, cconj(b)), w);
-    cf e2 = cadd(b, cconj(a));
-    cf o2 = cmul(csub(b, cconj(a)), w);
-    zk = {e1.x - o1.y, e1.y + o1.x};
-    zmk = {e2.x + o2.y, e2.y - o2.x};
+// packed inputs Z[k] (zk) and Z[M-k] (zmk), 0 < k < M: with E = a + conj(b)
+// and O = conj(w) (a - conj(b)), E + i O and conj(E - i O).
+template <class C>
+HD void c2r_pre_vals(C a, C b, C w, C& zk, C& zmk) {
+    const C e = cadd_conj(a, b), o = cmulc(csub_conj(a, b), w);
+    zk = caddi(e, o);
+    zmk = conj_subi(e, o);
 }
 
 }  // namespace hr

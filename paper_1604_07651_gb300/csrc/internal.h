@@ -20,6 +20,8 @@ struct FftPlan {            // radix schedule of one FFT length
     int rad[8];             // radix of each stage / pass
     int st[8];              // column plans (decimation in frequency): stride of each pass
     int tw[8];              // column plans: offset of each pass's twiddles in the table
+    int lst[8];             // log2 of the strides (powers of two)
+    int ntw;                // twiddle entries of all passes
 };
 
 // Lattice position of one gather sample, computed once per plan in FP64:
@@ -48,9 +50,12 @@ struct PieceDev {
     int Ntheta, Nrho, Ptheta, Prho;
     int ntaps;              // B-spline taps per axis: 4 (cubic) or 6 (quintic)
     int k1max, k2max;
-    int CB;                 // spectrum columns per block of the blocked layout
-    int nkb;                // number of column blocks: ceil((k2max+1)/CB)
-    int R;                  // lattice rows per band of the row kernels
+    int nkb;                // number of column blocks (two spectrum columns each): ceil((k2max+1)/2)
+    int C;                  // column blocks per CTA of the column pass
+    int nkg;                // its CTAs: ceil(nkb/C)
+    int sp;                 // lattice rows between the column blocks of spec (Ntheta, padded)
+    int lp;                 // row pitch of lat, floats: Nrho rounded up to 4
+    int Re;                 // lattice rows per band of the row kernels (even: they go in pairs)
     int nbands;
     // samples of the gather
     int Nt, Nx;
@@ -77,16 +82,18 @@ struct PieceDev {
     const float2* colw2;    // [ncol] theta tap weights 4 and 5 (six taps only; else null)
     const int* colm0;       // [ncol] first theta tap of each column
     const float* colscale;  // [ncol] output scale 2 X cos(psi) / a
-    const cf* K;            // [nkb][k1max+1][CB] kernel spectrum (normalised)
-    const cf* twM;          // pass twiddle tables of the row FFT pair (length Prho/2)
-    const int* rpos;        // [Prho/2] position of each frequency after the forward row passes
+    const float4* K;        // [nkb][k1max+2] kernel spectrum (normalised), two columns: (re0, re1, im0, im1); ends with a zero
+    const float4* twM;      // pass twiddle tables of the row FFT pair (length Prho/2), entries (wr, wr, wi, wi)
+    const int* rpos;        // [Prho/2] position (pad16) of each frequency after the forward row passes, for lengths
+                            // that are no multiple of 16
     const cf* twP;          // [Prho/2+1] exp(-2 pi i k / Prho)
-    const cf* twT;          // pass twiddle tables of the column FFT pair (length Ptheta), twT_len entries
-    int twT_len;            // entries of twT, a multiple of 2 (16-byte copies)
+    const float4* twT;      // pass twiddle tables of the column FFT pair (length Ptheta), entries (wr, wr, wi, wi)
     FftPlan fftM;           // row FFT (length Prho/2)
     FftPlan fftT;           // column FFT (length Ptheta)
-    float* lat;             // [Ntheta][Nrho] real lattice (Q forward, G' adjoint)
-    cf* spec;               // [nkb][Ntheta][CB] half spectrum of the lattice rows (in-place column pass)
+    float* lat;             // [Ntheta][lp] real lattice (Q forward, G' adjoint)
+    float4* spec;           // [nkb][sp] half spectrum of the lattice rows, two columns (2 kb, 2 kb + 1) per
+                            // element: (re0, re1, im0, im1) from the row FFT, and (im0, im1, re0, re1) once
+                            // the column pass has run (in place)
     float* prof;            // [ncol][hpitch] rho profiles of the output columns (adjoint)
     int hpitch;             // row pitch of prof, floats, multiple of 4
     long long f_off;        // element offset of this gather in packed gather buffers (0: single plan)
@@ -129,28 +136,34 @@ constexpr int kMaxBandRows = 6;
 // first descriptor's); another number than 4 or 6 returns
 // cudaErrorInvalidValue.
 int launch_grid_tiles(const PieceDev* P, int n, const float* f, void* stream);
-int launch_rows_r2c(const PieceDev* P, int n, void* stream);
-int launch_band_rows(const PieceDev* P, int n, void* stream);
+int launch_rows_r2c(const PieceDev* P, int n, int tpb, void* stream);
+int launch_band_rows(const PieceDev* P, int n, int tpb, void* stream);
 int launch_colconv(const PieceDev* P, int n, int adjoint, void* stream);
-int launch_rows_c2r(const PieceDev* P, int n, void* stream);
+int launch_rows_c2r(const PieceDev* P, int n, int tpb, void* stream);
+// Threads of a row-kernel CTA for one launch over the n pieces.
+int rows_threads(const PieceDev* P, int n, size_t smem);
+// Most pairs of rows a band of the piece may hold.
+int max_row_pairs(const PieceDev& P, size_t smem_max);
 // The same stages over a device-resident batch: `nblocks` blocks, map in S,
 // `smem` the largest dynamic shared memory any piece of the launch needs.
 int launch_grid_tiles_dev(const DevBatch& S, int nblocks, int ntaps, const void* f, int in_type, void* stream);
-int launch_rows_r2c_dev(const DevBatch& S, int nblocks, size_t smem, void* stream);
-int launch_band_rows_dev(const DevBatch& S, int nblocks, int ntaps, size_t smem, void* stream);
-// x256: every piece of the launch takes the compile-time column pass
-// (colconv_all_x256), which runs at fewer threads per CTA.
-int launch_colconv_dev(const DevBatch& S, int nblocks, size_t smem, bool x256, int adjoint, void* stream);
-bool colconv_all_x256(const PieceDev* P, int n);
-int launch_rows_c2r_dev(const DevBatch& S, int nblocks, size_t smem, void* stream);
+int launch_rows_r2c_dev(const DevBatch& S, int nblocks, int tpb, size_t smem, void* stream);
+int launch_band_rows_dev(const DevBatch& S, int nblocks, int ntaps, int tpb, size_t smem, void* stream);
+int launch_colconv_dev(const DevBatch& S, int nblocks, size_t smem, int adjoint, void* stream);
+// Column blocks per CTA (C, nkg) of every piece of one launch: as many as
+// give the CTA's threads a butterfly each, but no fewer than two CTAs per SM
+// (304) over the launch, so that a small gather still spreads over the chip.
+void set_col_groups(PieceDev* P, int n);
+int launch_rows_c2r_dev(const DevBatch& S, int nblocks, int tpb, size_t smem, void* stream);
 // Output interpolation: one CTA per output column; cmap[b] = (first piece,
 // number of time pieces, column l, 0) in `pieces` (device), or, when
 // np_all > 0 (one gather, one slowness piece of np_all time pieces, ntau_all
 // outputs per column), column b of pieces[0..np_all). np_max: the largest
 // number of time pieces of a column (<= kMaxColPieces); shared memory
 // np_max * nrho_max floats.
+// (rounded up to 16 bytes per piece within `limit`, interp_smem_limit).
 int launch_interp_columns(const PieceDev* pieces, const int4* cmap, int ncols, int nrho_max, int np_max,
-                          int ntau_all, int np_all, int ntaps, float* g, void* stream);
+                          int ntau_all, int np_all, int ntaps, size_t limit, float* g, void* stream);
 // Adjoint column profiles of every time piece of a column at once, one CTA
 // per output column (cmap / np_all / shared memory as the interpolation's).
 int launch_col_profiles_cols(const PieceDev* pieces, const int4* cmap, int ncols, int nrho_max, int np_max,
@@ -172,7 +185,6 @@ int launch_direct_fwd(const float* f, float* g, int Nt, int Nx, int Ntau, int Nq
                       double dx, double tau0, double dtau, double qmin, double dq, void* stream);
 int launch_direct_adj(const float* g, float* f, int Nt, int Nx, int Ntau, int Nq, double dt,
                       double dx, double tau0, double dtau, double qmin, double dq, void* stream);
-size_t scatter_smem_bytes(const PieceDev& P);   // = rows_smem_bytes
 
 // Forward transform of a plan with every work buffer carved out of the
 // caller-given device area `work` (256-byte aligned, `bytes` long) instead of

@@ -27,350 +27,13 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <mutex>
-#include <vector>
 
-#include "internal.h"
+#include "device.cuh"
 
 namespace hr {
 
-__device__ __forceinline__ cf ldcf(const cf* p) {
-    float2 v = __ldg(reinterpret_cast<const float2*>(p));
-    return {v.x, v.y};
-}
-// --------------------------------------------------------------------------
-// Row kernels: scatter into a band of lattice rows, then real FFT of the rows.
-// Shared memory: [R][Prho] floats (rows, viewed as [R][M] complex); the FFT
-// works in place.
-// --------------------------------------------------------------------------
-
-extern __shared__ __align__(16) float smem_f[];
-
-// Piece of this block in a batched launch, and the block's index within it:
-// from the descriptors passed as a kernel parameter (up to kMaxBatch pieces)
-// or from a device-resident batch (any number of pieces of many gathers).
-__device__ __forceinline__ int batch_piece(const PieceBatch& B, int& bx) {
-    int pi = 0;
-#pragma unroll
-    for (int k = 1; k < kMaxBatch; ++k)
-        if (k < B.n && (int)blockIdx.x >= B.first[k]) pi = k;
-    bx = (int)blockIdx.x - B.first[pi];
-    return pi;
-}
-__device__ __forceinline__ const PieceDev& piece_of(const PieceBatch& B, int& bx) { return B.p[batch_piece(B, bx)]; }
-__device__ __forceinline__ const PieceDev& piece_of(const DevBatch& B, int& bx) {
-    const int2 m = __ldg(B.map + blockIdx.x);
-    bx = m.y;
-    return B.p[m.x];
-}
-
-// Dynamic shared memory of the launch: the row and column kernels check it
-// against what their piece needs and leave the block untouched (never write
-// past it) if a launch gave too little.
-__device__ __forceinline__ unsigned dyn_smem_bytes() {
-    unsigned r;
-    asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(r));
-    return r;
-}
-
 __device__ __forceinline__ float load_in(const float* p) { return __ldg(p); }
 __device__ __forceinline__ float load_in(const __nv_bfloat16* p) { return __bfloat162float(__ldg(p)); }
-
-// Real sample n of a row buffer (stored as complex pairs in the sw layout).
-__device__ __forceinline__ int swr(int n) { return 2 * sw(n >> 1) + (n & 1); }
-
-// Row transforms: the real FFT of a lattice row of length Prho (first half
-// of Eq. (7)/(16)) as a complex FFT of the M = Prho / 2 packed pairs
-// z[n] = x[2n] + i x[2n+1], and its inverse, by the in-place decimation in
-// frequency / time of the column pass (dif_plan of M: P.fftM, twiddles
-// P.twM). The forward leaves Z in digit-reversed order; the real-FFT
-// post-processing reads Z[k] and Z[M - k] at their positions (P.rpos), and
-// the inverse's pre-processing writes the packed pairs straight to theirs.
-// One row butterfly per thread, the band's rows back to back in shared
-// memory ([R][M] complex, element i of a row at sw(i)), one barrier per pass.
-// Stride between the band's rows in shared memory, in complex elements: one
-// element of padding, so that the same position of the band's rows falls in
-// different banks (M is a multiple of 16).
-__host__ __device__ __forceinline__ int row_stride(int M) { return M + 1; }
-// Shared memory of the row kernels: R rows of row_stride(Prho / 2) complex.
-__host__ __device__ __forceinline__ size_t rows_smem(const PieceDev& P) {
-    return (size_t)P.R * row_stride(P.Prho / 2) * sizeof(cf);
-}
-
-template <int R>
-__device__ __forceinline__ void row_fwd(cf x[R], const cf* __restrict__ T, int S, int m) {
-    dft_small<R>(x, -1);
-    if (S > 1) {
-#pragma unroll
-        for (int k = 1; k < R; ++k) x[k] = cmul(x[k], ldcf(T + (k - 1) * S + m));
-    }
-}
-template <int R>
-__device__ __forceinline__ void row_inv(cf x[R], const cf* __restrict__ T, int S, int m) {
-    if (S > 1) {
-#pragma unroll
-        for (int k = 1; k < R; ++k) x[k] = cmulc(x[k], ldcf(T + (k - 1) * S + m));
-    }
-    dft_small<R>(x, +1);
-}
-
-// One pass over every row of the band, in place in shared memory.
-template <int R, bool INV>
-__device__ __forceinline__ void rows_pass(cf* X, int M, int nrows, int S, const cf* __restrict__ T) {
-    const int nb = M / R, tot = nb * nrows;
-    const float inv_nb = 1.0f / (float)nb, invS = 1.0f / (float)S;
-    for (int idx = threadIdx.x; idx < tot; idx += blockDim.x) {
-        const int row = (int)(((float)idx + 0.5f) * inv_nb);   // exact for idx < 2^22
-        const int b = idx - row * nb;
-        const int q = (int)(((float)b + 0.5f) * invS);
-        const int m = b - q * S;
-        const int base = q * S * R + m;
-        cf* Z = X + row * row_stride(M);
-        cf x[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) x[r] = Z[sw(base + r * S)];
-        if (INV) row_inv<R>(x, T, S, m);
-        else row_fwd<R>(x, T, S, m);
-#pragma unroll
-        for (int r = 0; r < R; ++r) Z[sw(base + r * S)] = x[r];
-    }
-}
-
-// Forward pass 0 reading the band's lattice rows (Nr reals each, zero padded)
-// from global memory.
-template <int R>
-__device__ __forceinline__ void rows_first_lat(cf* X, const float* __restrict__ lat, int Nr, int M, int nrows, int S,
-                                               const cf* __restrict__ T) {
-    const int tot = S * nrows;
-    const float invS = 1.0f / (float)S;
-    for (int idx = threadIdx.x; idx < tot; idx += blockDim.x) {
-        const int row = (int)(((float)idx + 0.5f) * invS);
-        const int m = idx - row * S;
-        const float* src = lat + (size_t)row * Nr;
-        cf x[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int n2 = 2 * (m + r * S);
-            x[r].x = n2 < Nr ? __ldg(src + n2) : 0.f;
-            x[r].y = n2 + 1 < Nr ? __ldg(src + n2 + 1) : 0.f;
-        }
-        row_fwd<R>(x, T, S, m);
-        cf* Z = X + row * row_stride(M);
-#pragma unroll
-        for (int r = 0; r < R; ++r) Z[sw(m + r * S)] = x[r];
-    }
-}
-
-// Inverse pass 0 writing the band's lattice rows (first Nr reals) to global
-// memory.
-template <int R>
-__device__ __forceinline__ void rows_last_lat(const cf* X, float* lat, int Nr, int M, int nrows, int S,
-                                              const cf* __restrict__ T) {
-    const int tot = S * nrows;
-    const float invS = 1.0f / (float)S;
-    for (int idx = threadIdx.x; idx < tot; idx += blockDim.x) {
-        const int row = (int)(((float)idx + 0.5f) * invS);
-        const int m = idx - row * S;
-        const cf* Z = X + row * row_stride(M);
-        cf x[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) x[r] = Z[sw(m + r * S)];
-        row_inv<R>(x, T, S, m);
-        float* dst = lat + (size_t)row * Nr;
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int n2 = 2 * (m + r * S);
-            if (n2 < Nr) dst[n2] = x[r].x;
-            if (n2 + 1 < Nr) dst[n2 + 1] = x[r].y;
-        }
-    }
-}
-
-#define HR_RADIX_CASES(CALL) \
-    case 16: CALL(16); break; \
-    case 12: CALL(12); break; \
-    case 10: CALL(10); break; \
-    case 9: CALL(9); break;   \
-    case 8: CALL(8); break;   \
-    case 6: CALL(6); break;   \
-    case 5: CALL(5); break;   \
-    case 4: CALL(4); break;   \
-    case 3: CALL(3); break;   \
-    default: CALL(2); break;
-
-// The same passes for the row lengths M = R0 * 256 with radices R0, 16, 16
-// (the plans of the 2048^2 and 4096^2 workloads), every length, stride and
-// count a compile-time constant (the index arithmetic folds to shifts and
-// constant divisions). Same arithmetic as the general passes.
-template <int R, int S, int M, bool INV>
-__device__ __forceinline__ void rows_pass_c(cf* X, int nrows, const cf* __restrict__ T) {
-    constexpr int nb = M / R;
-    const int tot = nb * nrows;
-    for (int idx = threadIdx.x; idx < tot; idx += blockDim.x) {
-        const int row = idx / nb;
-        const int b = idx - row * nb;
-        const int q = b / S, m = b - q * S;
-        const int base = q * S * R + m;
-        cf* Z = X + row * row_stride(M);
-        cf x[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) x[r] = Z[sw(base + r * S)];
-        if (INV) row_inv<R>(x, T, S, m);
-        else row_fwd<R>(x, T, S, m);
-#pragma unroll
-        for (int r = 0; r < R; ++r) Z[sw(base + r * S)] = x[r];
-    }
-}
-template <int R0>
-__device__ __forceinline__ void rows_first_lat_c(cf* X, const float* __restrict__ lat, int Nr, int nrows,
-                                                 const cf* __restrict__ T) {
-    constexpr int S = 256, M = R0 * 256;
-    const int tot = S * nrows;
-    for (int idx = threadIdx.x; idx < tot; idx += blockDim.x) {
-        const int row = idx / S, m = idx % S;
-        const float* src = lat + (size_t)row * Nr;
-        cf x[R0];
-#pragma unroll
-        for (int r = 0; r < R0; ++r) {
-            const int n2 = 2 * (m + r * S);
-            x[r].x = n2 < Nr ? __ldg(src + n2) : 0.f;
-            x[r].y = n2 + 1 < Nr ? __ldg(src + n2 + 1) : 0.f;
-        }
-        row_fwd<R0>(x, T, S, m);
-        cf* Z = X + row * row_stride(M);
-#pragma unroll
-        for (int r = 0; r < R0; ++r) Z[sw(m + r * S)] = x[r];
-    }
-}
-template <int R0>
-__device__ __forceinline__ void rows_last_lat_c(const cf* X, float* lat, int Nr, int nrows, const cf* __restrict__ T) {
-    constexpr int S = 256, M = R0 * 256;
-    const int tot = S * nrows;
-    for (int idx = threadIdx.x; idx < tot; idx += blockDim.x) {
-        const int row = idx / S, m = idx % S;
-        const cf* Z = X + row * row_stride(M);
-        cf x[R0];
-#pragma unroll
-        for (int r = 0; r < R0; ++r) x[r] = Z[sw(m + r * S)];
-        row_inv<R0>(x, T, S, m);
-        float* dst = lat + (size_t)row * Nr;
-#pragma unroll
-        for (int r = 0; r < R0; ++r) {
-            const int n2 = 2 * (m + r * S);
-            if (n2 < Nr) dst[n2] = x[r].x;
-            if (n2 + 1 < Nr) dst[n2 + 1] = x[r].y;
-        }
-    }
-}
-// R0 of a plan of length R0 * 256 with radices R0, 16, 16, else 0.
-__device__ __forceinline__ int plan_x256(const FftPlan& fp) {
-    return (fp.nst == 3 && fp.st[0] == 256 && fp.rad[1] == 16 && fp.rad[2] == 16) ? fp.rad[0] : 0;
-}
-#define HR_X256_CASES(CALL) \
-    case 2: CALL(2); break;  \
-    case 3: CALL(3); break;  \
-    case 4: CALL(4); break;  \
-    case 5: CALL(5); break;  \
-    case 6: CALL(6); break;  \
-    case 8: CALL(8); break;  \
-    case 9: CALL(9); break;  \
-    case 10: CALL(10); break; \
-    case 12: CALL(12); break;
-
-// Forward passes p0 .. s-1 in shared memory (p0 = 1 after rows_first_lat).
-__device__ __forceinline__ void rows_fwd_passes(cf* X, int M, int nrows, const FftPlan& fp, const cf* T, int p0) {
-    switch (plan_x256(fp)) {
-#define HR_RX(R0)                                                                    \
-    if (p0 == 0) {                                                                   \
-        rows_pass_c<R0, 256, R0 * 256, false>(X, nrows, T);                          \
-        __syncthreads();                                                             \
-    }                                                                                \
-    rows_pass_c<16, 16, R0 * 256, false>(X, nrows, T + fp.tw[1]);                    \
-    __syncthreads();                                                                 \
-    rows_pass_c<16, 1, R0 * 256, false>(X, nrows, T);                                \
-    __syncthreads();                                                                 \
-    return;
-        HR_X256_CASES(HR_RX)
-#undef HR_RX
-        default: break;
-    }
-    for (int p = p0; p < fp.nst; ++p) {
-#define HR_RF(RR) rows_pass<RR, false>(X, M, nrows, fp.st[p], T + fp.tw[p])
-        switch (fp.rad[p]) { HR_RADIX_CASES(HR_RF) }
-#undef HR_RF
-        __syncthreads();
-    }
-}
-
-// Real-FFT post-processing of the band's transformed rows (digit-reversed in
-// shared memory) into the half spectrum, bins k <= k2max, blocked layout.
-__device__ __forceinline__ void rows_post(const PieceDev& P, const cf* Z0, int mb, int nrows) {
-    cf* __restrict__ spec = P.spec;
-    const int M = P.Prho / 2;
-    const int nk = P.k2max + 1;
-    const int per_kb = nrows * 2;                 // (row, c) of a column block (CB = 2), c fastest
-    const int total = P.nkb * per_kb;
-    const float inv_per_kb = 1.0f / (float)per_kb;
-    for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
-        const int kb = (int)(((float)idx + 0.5f) * inv_per_kb);   // exact for idx < 2^22
-        const int rem = idx - kb * per_kb;
-        const int m = rem >> 1;
-        const int c = rem & 1;
-        const int k = kb * 2 + c;
-        cf X = {0.f, 0.f};
-        if (k < nk)
-            X = r2c_post_at(Z0 + m * row_stride(M), sw(__ldg(P.rpos + k)), sw(__ldg(P.rpos + (k == 0 ? 0 : M - k))), k,
-                            P.twP);
-        spec[((size_t)kb * P.Ntheta + (mb + m)) * 2 + c] = X;
-    }
-}
-
-// Inverse: the real-FFT pre-processing of the band's half-spectrum rows
-// (bins above k2max are zero), pairs (k, M - k) for 0 <= k <= M/2, written to
-// their digit-reversed positions in shared memory.
-__device__ __forceinline__ void rows_pre(const PieceDev& P, cf* X, int mb, int nrows) {
-    const cf* __restrict__ spec = P.spec;
-    const int M = P.Prho / 2, half = M / 2;
-    const int nk = P.k2max + 1;
-    const int per_kb = nrows * 2;                 // (row, c) of a column block, c fastest
-    const int total = (half / 2 + 1) * per_kb;    // k = 2 kb + c <= half
-    constexpr int U = 4;                          // pairs per thread whose spectrum loads go out together
-    const float inv_per_kb = 1.0f / (float)per_kb;
-    for (int i0 = threadIdx.x; i0 < total; i0 += U * blockDim.x) {
-        cf a[U], b[U];
-        int kk[U], mm[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int idx = i0 + u * (int)blockDim.x;
-            const int kb = (int)(((float)idx + 0.5f) * inv_per_kb);   // exact for idx < 2^22
-            const int rem = idx - kb * per_kb;
-            const int m = rem >> 1;
-            const int k = 2 * kb + (rem & 1);
-            kk[u] = idx < total && k <= half ? k : -1;
-            mm[u] = m;
-            a[u] = b[u] = cf{0.f, 0.f};
-            if (kk[u] < 0) continue;
-            const size_t rowoff = (size_t)(mb + m) * 2;
-            const int k2 = M - k;
-            if (k < nk) a[u] = ldcf(spec + (size_t)(k >> 1) * P.Ntheta * 2 + rowoff + (k & 1));
-            if (k > 0 && k2 < nk) b[u] = ldcf(spec + (size_t)(k2 >> 1) * P.Ntheta * 2 + rowoff + (k2 & 1));
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int k = kk[u];
-            if (k < 0) continue;
-            cf* Z = X + mm[u] * row_stride(M);
-            if (k == 0) {
-                Z[sw(__ldg(P.rpos))] = c2r_pre_dc(a[u]);
-                continue;
-            }
-            cf zk, zmk;
-            c2r_pre_vals(a[u], b[u], ldcf(P.twP + k), zk, zmk);
-            Z[sw(__ldg(P.rpos + k))] = zk;
-            Z[sw(__ldg(P.rpos + M - k))] = zmk;
-        }
-    }
-}
 
 // Shared gridding tile: the kTileRows x kTileCols cells plus a halo of
 // NT - 1 cells on every side (NT taps per axis: 4 cubic, 6 quintic), so that
@@ -515,7 +178,7 @@ __device__ __forceinline__ void grid_merge_split(const PieceDev& P, int4 us, int
     float* slot0 = P.slots + (size_t)us.x * kCells;
     for (int i = threadIdx.x; i < kCells; i += blockDim.x) slot0[(size_t)us.z * kCells + i] = value(i);
     __syncthreads();
-    int* counter = reinterpret_cast<int*>(P.lat + (size_t)P.Ntheta * P.Nrho) + us.w;
+    int* counter = reinterpret_cast<int*>(P.lat + (size_t)P.Ntheta * P.lp) + us.w;
     if (threadIdx.x == 0) {
         __threadfence();
         const int last = atomicAdd(counter, 1) == us.y - 1;
@@ -544,7 +207,7 @@ __device__ __forceinline__ void grid_merge_split(const PieceDev& P, int4 us, int
     for (int j = 0; j < kPer; ++j) {
         const int i = threadIdx.x + j * kUnitChunks;
         const int m = i / kTileCols, n = i - m * kTileCols;
-        if (m < nr && n < nc) P.lat[(size_t)(m_lo + m) * P.Nrho + n_lo + n] = acc[j];
+        if (m < nr && n < nc) P.lat[(size_t)(m_lo + m) * P.lp + n_lo + n] = acc[j];
     }
     if (threadIdx.x == 0) *counter = 0;
 }
@@ -599,7 +262,7 @@ __global__ void __launch_bounds__(kUnitChunks, NT == 4 ? 4 : 2) k_grid_tiles(con
         } else if (fill != 0.f) {
             for (int i = threadIdx.x; i < kTileRows * kTileCols; i += blockDim.x) {
                 const int m = i / kTileCols, n = i - m * kTileCols;
-                if (m < nr && n < nc) P.lat[(size_t)(m_lo + m) * P.Nrho + n_lo + n] = fill;
+                if (m < nr && n < nc) P.lat[(size_t)(m_lo + m) * P.lp + n_lo + n] = fill;
             }
         }
         return;
@@ -656,35 +319,8 @@ __global__ void __launch_bounds__(kUnitChunks, NT == 4 ? 4 : 2) k_grid_tiles(con
     for (int i = threadIdx.x; i < kTileRows * kTileCols; i += blockDim.x) {   // the tile's only unit
         const int m = i / kTileCols, n = i - m * kTileCols;
         const int t = tile[(m + Tile::halo) * Tile::pitch + n + Tile::halo];
-        if (t != 0 && m < nr && n < nc) P.lat[(size_t)(m_lo + m) * P.Nrho + n_lo + n] = sc.down(t);
+        if (t != 0 && m < nr && n < nc) P.lat[(size_t)(m_lo + m) * P.lp + n_lo + n] = sc.down(t);
     }
-}
-
-// Real FFT of a band of lattice rows (P.lat, zero-padded to Prho) into the
-// half spectrum (first half of Eq. (7)/(16)): pass 0 reads the rows from
-// global memory.
-template <class Src>
-__global__ void __launch_bounds__(512, 2) k_rows_r2c(const __grid_constant__ Src B) {
-    int bx;
-    const PieceDev& P = piece_of(B, bx);
-    if (P.CB != 2 || rows_smem(P) > dyn_smem_bytes()) return;
-    const int mb = bx * P.R;
-    const int nrows = min(P.R, P.Ntheta - mb);
-    const int M = P.Prho / 2;
-    cf* X = reinterpret_cast<cf*>(smem_f);
-    const FftPlan& fp = P.fftM;
-    switch (plan_x256(fp)) {
-#define HR_RL(R0) rows_first_lat_c<R0>(X, P.lat + (size_t)mb * P.Nrho, P.Nrho, nrows, P.twM); break;
-        HR_X256_CASES(HR_RL)
-#undef HR_RL
-        default:
-#define HR_RL(RR) rows_first_lat<RR>(X, P.lat + (size_t)mb * P.Nrho, P.Nrho, M, nrows, fp.st[0], P.twM)
-            switch (fp.rad[0]) { HR_RADIX_CASES(HR_RL) }
-#undef HR_RL
-    }
-    __syncthreads();
-    rows_fwd_passes(X, M, nrows, fp, P.twM, 1);
-    rows_post(P, X, mb, nrows);
 }
 
 // Adjoint of the output interpolation (transpose of Eq. (17)), separated
@@ -834,398 +470,6 @@ __global__ void __launch_bounds__(256) k_col_profiles_cols(const PieceDev* __res
     }
 }
 
-// One band of R <= kMaxBandRows lattice rows: G' rows from the profiles of
-// the band's candidate columns (NT theta taps of each column from the plan),
-// then the row FFT into the half spectrum. Each thread owns four rho cells
-// of every row of the band and sums the columns in order in registers.
-template <class Src, int NT>
-__global__ void __launch_bounds__(512, 2) k_band_rows(const __grid_constant__ Src B) {
-    int band;
-    const PieceDev& P = piece_of(B, band);
-    if (P.CB != 2 || rows_smem(P) > dyn_smem_bytes()) return;
-    const float* __restrict__ h = P.prof;
-    const int hp = P.hpitch;
-    const int mb = band * P.R;
-    const int nrows = min(P.R, P.Ntheta - mb);
-    const int2 lr = __ldg(P.lband + band);
-    const int Pr = P.Prho;
-    for (int n4 = threadIdx.x; n4 < Pr / 4; n4 += blockDim.x) {
-        float4 acc[kMaxBandRows];
-#pragma unroll
-        for (int r = 0; r < kMaxBandRows; ++r) acc[r] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (4 * n4 < hp) {
-#pragma unroll 4
-            for (int l = lr.x; l <= lr.y; ++l) {
-                const int lc = l - P.l_lo;
-                const int a0 = mb - __ldg(P.colm0 + lc);     // tap of the band's first row
-                const float4 w4 = __ldg(P.colw + lc);
-                const float2 w2 = NT > 4 ? __ldg(P.colw2 + lc) : make_float2(0.f, 0.f);
-                const float4 hv = __ldg(reinterpret_cast<const float4*>(h + (size_t)lc * hp) + n4);
-#pragma unroll
-                for (int r = 0; r < kMaxBandRows; ++r) {
-                    const int a = a0 + r;
-                    if (r < nrows && a >= 0 && a < NT) {
-                        const float w = a == 0 ? w4.x : a == 1 ? w4.y : a == 2 ? w4.z : a == 3 ? w4.w
-                                      : a == 4 ? w2.x : w2.y;
-                        acc[r].x = fmaf(w, hv.x, acc[r].x);
-                        acc[r].y = fmaf(w, hv.y, acc[r].y);
-                        acc[r].z = fmaf(w, hv.z, acc[r].z);
-                        acc[r].w = fmaf(w, hv.w, acc[r].w);
-                    }
-                }
-            }
-        }
-#pragma unroll
-        for (int r = 0; r < kMaxBandRows; ++r) {
-            if (r < nrows) {
-                float* row = smem_f + r * 2 * row_stride(Pr / 2);
-                const int n = 4 * n4;
-                row[swr(n)] = acc[r].x;
-                row[swr(n + 1)] = acc[r].y;
-                row[swr(n + 2)] = acc[r].z;
-                row[swr(n + 3)] = acc[r].w;
-            }
-        }
-    }
-    __syncthreads();
-    rows_fwd_passes(reinterpret_cast<cf*>(smem_f), P.Prho / 2, nrows, P.fftM, P.twM, 0);
-    rows_post(P, reinterpret_cast<const cf*>(smem_f), mb, nrows);
-}
-
-// --------------------------------------------------------------------------
-// Column pass: FFT along theta, product with K (or conj K), inverse FFT
-// (Eq. (16)-(17)). One CTA of kColThreads threads per block of two spectrum
-// columns, which the blocked layout [kb][m][2] stores as one 16-byte row per
-// lattice row; thread pairs (2 t, 2 t + 1) take the same butterfly of the two
-// columns, so every shared and global access of a pair is one 16-byte word
-// (shared buffer [Ptheta] of 16-byte elements, swizzled by swc). One column
-// per thread keeps a radix-16 butterfly in 64 registers; three CTAs (30
-// warps) per SM hide the pass latencies (measured at 2048^2: 49.5 us against
-// 54.7 us at 512 threads and two CTAs per SM, 59 us at 384 threads; earlier,
-// both columns per thread at 256 threads 90 us, that at one CTA per SM 112).
-// The column block's slice of K and the pass twiddle tables are copied into
-// shared memory (cp.async) while pass 0 runs.
-//
-// The pair runs in place by decimation in frequency / time (dif_plan):
-//   pass 0        reads the column block's Ntheta rows straight from global
-//                 memory (the zero padding is never loaded) and writes
-//                 shared memory;
-//   passes 1..    forward passes in shared memory, one barrier each;
-//   last pass     (stride 1) forward butterfly, product with K at each
-//                 element's frequency (digit-reversed order: no reordering),
-//                 inverse butterfly, all in registers;
-//   back down     inverse passes, the last one writing only the Ntheta rows
-//                 back to global memory.
-// --------------------------------------------------------------------------
-// Threads of a column-pass CTA: two per butterfly of the two columns. 320
-// keeps the radix-16 passes of the R0 * 256 lengths (144 or 160 butterflies
-// per column) 90-100 % busy, with three CTAs per SM; launches with a piece of
-// another length (the general passes, all twiddle tables in shared memory)
-// take 512 threads and two CTAs per SM.
-constexpr int kColThreads = 320;
-constexpr int kColThreadsGeneral = 512;
-// 16-byte asynchronous copies global -> shared (cp.async; the completion
-// wait is the hardware's, no spin loop).
-__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gmem_src) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() {
-    asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
-}
-
-template <int R>
-__device__ __forceinline__ void c1_fwd(cf x[R], const cf* T, int S, int m) {
-    dft_small<R>(x, -1);
-    if (S > 1) {
-#pragma unroll
-        for (int k = 1; k < R; ++k) x[k] = cmul(x[k], T[(k - 1) * S + m]);
-    }
-}
-template <int R>
-__device__ __forceinline__ void c1_inv(cf x[R], const cf* T, int S, int m) {
-    if (S > 1) {
-#pragma unroll
-        for (int k = 1; k < R; ++k) x[k] = cmulc(x[k], T[(k - 1) * S + m]);
-    }
-    dft_small<R>(x, +1);
-}
-template <int R>
-__device__ __forceinline__ void c1_ld(const cf* A, int base, int S, int c, cf x[R]) {
-#pragma unroll
-    for (int r = 0; r < R; ++r) x[r] = A[2 * swc(base + r * S) + c];
-}
-template <int R>
-__device__ __forceinline__ void c1_st(cf* A, int base, int S, int c, const cf x[R]) {
-#pragma unroll
-    for (int r = 0; r < R; ++r) A[2 * swc(base + r * S) + c] = x[r];
-}
-template <int R>
-__device__ __forceinline__ void c1_first(cf* A, const cf* __restrict__ col, int Nth, int S, const cf* T, int t, int nt, int c) {
-    for (int m = t; m < S; m += nt) {
-        cf x[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int row = m + r * S;
-            x[r] = row < Nth ? ldcf(col + 2 * row + c) : cf{0.f, 0.f};
-        }
-        c1_fwd<R>(x, T, S, m);
-        c1_st<R>(A, m, S, c, x);
-    }
-}
-template <int R>
-__device__ __forceinline__ void c1_last(const cf* A, cf* col, int Nth, int S, const cf* T, int t, int nt, int c) {
-    for (int m = t; m < S; m += nt) {
-        cf x[R];
-        c1_ld<R>(A, m, S, c, x);
-        c1_inv<R>(x, T, S, m);
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int row = m + r * S;
-            if (row < Nth) col[2 * row + c] = x[r];
-        }
-    }
-}
-template <int R, bool INV>
-__device__ __forceinline__ void c1_mid(cf* A, int n, int S, const cf* T, int t, int nt, int c) {
-    const int nb = n / R;
-    const float invS = 1.0f / (float)S;
-    for (int b = t; b < nb; b += nt) {
-        const int q = (int)(((float)b + 0.5f) * invS);
-        const int m = b - q * S;
-        const int base = q * S * R + m;
-        cf x[R];
-        c1_ld<R>(A, base, S, c, x);
-        if (INV) c1_inv<R>(x, T, S, m);
-        else c1_fwd<R>(x, T, S, m);
-        c1_st<R>(A, base, S, c, x);
-    }
-}
-template <int R>
-__device__ __forceinline__ void c1_kernel(cf* A, const FftPlan& fp, const cf* K, int k1n, int adjoint, int t, int nt, int c) {
-    const int n = fp.n, s = fp.nst;
-    const int nb = n / R;
-    for (int b = t; b < nb; b += nt) {
-        int fb = 0, w = 1, rem = b;
-        for (int p = 0; p + 1 < s; ++p) {
-            const int d = fp.st[p] / R;
-            const int k = (int)(((float)rem + 0.5f) / (float)d);
-            rem -= k * d;
-            fb += k * w;
-            w *= fp.rad[p];
-        }
-        cf x[R];
-        c1_ld<R>(A, b * R, 1, c, x);
-        dft_small<R>(x, -1);
-#pragma unroll
-        for (int k = 0; k < R; ++k) {
-            const int f = fb + nb * k;
-            const int kk = f <= n - f ? f : n - f;
-            if (kk < k1n) {
-                const cf kv = K[2 * kk + c];
-                x[k] = adjoint ? cmulc(x[k], kv) : cmul(x[k], kv);
-            } else {
-                x[k] = cf{0.f, 0.f};
-            }
-        }
-        dft_small<R>(x, +1);
-        c1_st<R>(A, b * R, 1, c, x);
-    }
-}
-
-// The pair for Ptheta = R0 * 256 (radices R0, 16, 16: the plans of the
-// 2048^2 workload) with every stride and count a compile-time constant: one
-// butterfly per thread and pass (256 threads per column), the stride-1
-// pass's first frequency b / 16 + R0 (b mod 16) without the general digit
-// loop. Same arithmetic as the general passes.
-template <int R0>
-__device__ __forceinline__ void c1_x256(cf* A, cf* col, int Nth, const cf* Tg, const cf* T1, const cf* K, int k1n,
-                                        int adjoint, int t, int nt, int c) {
-    constexpr int n = R0 * 256, nb = R0 * 16;
-    c1_first<R0>(A, col, Nth, 256, Tg, t, nt, c);
-    cp_async_wait_all();
-    __syncthreads();
-    for (int b = t; b < nb; b += nt) {
-        const int q = b >> 4, m = b & 15;
-        cf x[16];
-        c1_ld<16>(A, q * 256 + m, 16, c, x);
-        c1_fwd<16>(x, T1, 16, m);
-        c1_st<16>(A, q * 256 + m, 16, c, x);
-    }
-    __syncthreads();
-    for (int b = t; b < nb; b += nt) {
-        const int q = b >> 4, m = b & 15;
-        const int fb = q + R0 * m;
-        cf x[16];
-        c1_ld<16>(A, b * 16, 1, c, x);
-        // forward DFT, product with K, inverse DFT as conj(DFT(conj(.))):
-        // one DFT body run twice (half the code of the pass)
-#pragma unroll 1
-        for (int h = 0; h < 2; ++h) {
-            dft_small<16>(x, -1);
-            if (h == 0) {
-#pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    const int f = fb + nb * k;
-                    const int kk = f <= n - f ? f : n - f;
-                    if (kk < k1n) {
-                        const cf kv = K[2 * kk + c];
-                        x[k] = cconj(adjoint ? cmulc(x[k], kv) : cmul(x[k], kv));
-                    } else {
-                        x[k] = cf{0.f, 0.f};
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int k = 0; k < 16; ++k) x[k] = cconj(x[k]);
-            }
-        }
-        c1_st<16>(A, b * 16, 1, c, x);
-    }
-    __syncthreads();
-    for (int b = t; b < nb; b += nt) {
-        const int q = b >> 4, m = b & 15;
-        cf x[16];
-        c1_ld<16>(A, q * 256 + m, 16, c, x);
-        c1_inv<16>(x, T1, 16, m);
-        c1_st<16>(A, q * 256 + m, 16, c, x);
-    }
-    __syncthreads();
-    c1_last<R0>(A, col, Nth, 256, Tg, t, nt, c);
-}
-
-// R0 of a column plan that the compile-time pair c1_x256 serves, else 0.
-__host__ __device__ __forceinline__ int colconv_x256(const FftPlan& fp) {
-    if (fp.nst != 3 || fp.st[0] != 256 || fp.rad[1] != 16 || fp.rad[2] != 16) return 0;
-    const int r = fp.rad[0];
-    return (r == 5 || r == 6 || r == 8 || r == 9 || r == 10 || r == 12) ? r : 0;
-}
-
-// Shared memory of the column kernel: the column block [Ptheta] (16-byte
-// elements), its slice of K [k1max + 1] (16 bytes each), the twiddle tables
-// (twlen complex, a multiple of 2): all passes' tables, or for the
-// compile-time pair only the stride-16 pass's 240 (the first pass reads its
-// own from global memory), which lets three CTAs share an SM.
-constexpr int kX256Twiddles = 16 * 15;
-__host__ __device__ __forceinline__ size_t colconv_smem(int Pt, int k1n, int twlen) {
-    return ((size_t)Pt + k1n) * 16 + (size_t)twlen * 8;
-}
-__host__ __device__ __forceinline__ size_t colconv_smem(const PieceDev& P) {
-    return colconv_smem(P.Ptheta, P.k1max + 1, colconv_x256(P.fftT) ? kX256Twiddles : P.twT_len);
-}
-
-template <class Src, int TPB>
-__global__ void __launch_bounds__(TPB, TPB == kColThreads ? 3 : 2) k_colconv(const __grid_constant__ Src B, int adjoint) {
-    int kb;
-    const PieceDev& P = piece_of(B, kb);
-    const int Pt = P.Ptheta, Nth = P.Ntheta, k1n = P.k1max + 1;
-    if (P.CB != 2 || (P.twT_len & 1) || colconv_smem(P) > dyn_smem_bytes()) return;
-    const int x256 = colconv_x256(P.fftT);
-    float4* A4 = reinterpret_cast<float4*>(smem_f);
-    float4* Ks4 = A4 + Pt;
-    cf* Ts = reinterpret_cast<cf*>(Ks4 + k1n);
-    cf* A = reinterpret_cast<cf*>(A4);
-    const cf* K = reinterpret_cast<const cf*>(Ks4);
-    cf* col = P.spec + (size_t)kb * Nth * 2;
-    {
-        const float4* Kg = reinterpret_cast<const float4*>(P.K) + (size_t)kb * k1n;
-        for (int i = threadIdx.x; i < k1n; i += blockDim.x) cp_async16(Ks4 + i, Kg + i);
-        const float4* Tg = reinterpret_cast<const float4*>(P.twT + (x256 ? P.fftT.tw[1] : 0));
-        float4* T4 = reinterpret_cast<float4*>(Ts);
-        const int n4 = (x256 ? kX256Twiddles : P.twT_len) / 2;
-        for (int i = threadIdx.x; i < n4; i += blockDim.x) cp_async16(T4 + i, Tg + i);
-    }
-    const int c = threadIdx.x & 1, t = threadIdx.x >> 1, nt = blockDim.x >> 1;
-    const FftPlan& fp = P.fftT;
-    const int s = fp.nst;
-    const cf* T = Ts;
-    const int R0 = fp.rad[0], S0 = fp.st[0];
-    if (s == 1) {
-        for (int m = threadIdx.x; m < Pt; m += blockDim.x)
-            A4[swc(m)] = m < Nth ? __ldg(reinterpret_cast<const float4*>(col) + m) : make_float4(0.f, 0.f, 0.f, 0.f);
-        cp_async_wait_all();
-        __syncthreads();
-#define HR_K(RR) c1_kernel<RR>(A, fp, K, k1n, adjoint, t, nt, c)
-        switch (R0) { HR_RADIX_CASES(HR_K) }
-        __syncthreads();
-        for (int m = threadIdx.x; m < Nth; m += blockDim.x) reinterpret_cast<float4*>(col)[m] = A4[swc(m)];
-        return;
-    }
-    switch (x256) {
-        case 5: c1_x256<5>(A, col, Nth, P.twT, T, K, k1n, adjoint, t, nt, c); return;
-        case 6: c1_x256<6>(A, col, Nth, P.twT, T, K, k1n, adjoint, t, nt, c); return;
-        case 8: c1_x256<8>(A, col, Nth, P.twT, T, K, k1n, adjoint, t, nt, c); return;
-        case 9: c1_x256<9>(A, col, Nth, P.twT, T, K, k1n, adjoint, t, nt, c); return;
-        case 10: c1_x256<10>(A, col, Nth, P.twT, T, K, k1n, adjoint, t, nt, c); return;
-        case 12: c1_x256<12>(A, col, Nth, P.twT, T, K, k1n, adjoint, t, nt, c); return;
-        default: break;
-    }
-#define HR_FIRST(RR) c1_first<RR>(A, col, Nth, S0, P.twT, t, nt, c)
-    switch (R0) { HR_RADIX_CASES(HR_FIRST) }
-    cp_async_wait_all();
-    __syncthreads();
-    for (int p = 1; p + 1 < s; ++p) {
-#define HR_FWD(RR) c1_mid<RR, false>(A, Pt, fp.st[p], T + fp.tw[p], t, nt, c)
-        switch (fp.rad[p]) { HR_RADIX_CASES(HR_FWD) }
-        __syncthreads();
-    }
-    switch (fp.rad[s - 1]) { HR_RADIX_CASES(HR_K) }
-    __syncthreads();
-    for (int p = s - 2; p >= 1; --p) {
-#define HR_INV(RR) c1_mid<RR, true>(A, Pt, fp.st[p], T + fp.tw[p], t, nt, c)
-        switch (fp.rad[p]) { HR_RADIX_CASES(HR_INV) }
-        __syncthreads();
-    }
-#define HR_LAST(RR) c1_last<RR>(A, col, Nth, S0, T, t, nt, c)
-    switch (R0) { HR_RADIX_CASES(HR_LAST) }
-#undef HR_K
-#undef HR_FIRST
-#undef HR_FWD
-#undef HR_INV
-#undef HR_LAST
-}
-
-// --------------------------------------------------------------------------
-// Inverse real FFT of a band of rows from the half spectrum (bins <= k2max,
-// the rest zero) into the real lattice P.lat[Ntheta][Nrho]: the
-// pre-processing reads the spectrum from global memory, the last pass writes
-// the lattice rows.
-// --------------------------------------------------------------------------
-template <class Src>
-__global__ void __launch_bounds__(512, 2) k_rows_c2r(const __grid_constant__ Src B) {
-    int bx;
-    const PieceDev& P = piece_of(B, bx);
-    if (P.CB != 2 || rows_smem(P) > dyn_smem_bytes()) return;
-    const int mb = bx * P.R;
-    const int nrows = min(P.R, P.Ntheta - mb);
-    const int M = P.Prho / 2;
-    cf* X = reinterpret_cast<cf*>(smem_f);
-    const FftPlan& fp = P.fftM;
-    rows_pre(P, X, mb, nrows);
-    __syncthreads();
-    switch (plan_x256(fp)) {
-#define HR_CX(R0)                                                                    \
-    rows_pass_c<16, 1, R0 * 256, true>(X, nrows, P.twM);                             \
-    __syncthreads();                                                                 \
-    rows_pass_c<16, 16, R0 * 256, true>(X, nrows, P.twM + fp.tw[1]);                 \
-    __syncthreads();                                                                 \
-    rows_last_lat_c<R0>(X, P.lat + (size_t)mb * P.Nrho, P.Nrho, nrows, P.twM);       \
-    return;
-        HR_X256_CASES(HR_CX)
-#undef HR_CX
-        default: break;
-    }
-    for (int p = fp.nst - 1; p >= 1; --p) {
-#define HR_RI(RR) rows_pass<RR, true>(X, M, nrows, fp.st[p], P.twM + fp.tw[p])
-        switch (fp.rad[p]) { HR_RADIX_CASES(HR_RI) }
-#undef HR_RI
-        __syncthreads();
-    }
-#define HR_RW(RR) rows_last_lat<RR>(X, P.lat + (size_t)mb * P.Nrho, P.Nrho, M, nrows, fp.st[0], P.twM)
-    switch (fp.rad[0]) { HR_RADIX_CASES(HR_RW) }
-#undef HR_RW
-}
-
 // --------------------------------------------------------------------------
 // Gathers.
 // --------------------------------------------------------------------------
@@ -1252,20 +496,20 @@ __device__ __forceinline__ float taps_nt(const float* __restrict__ lat, int Nr, 
 // theta taps, so the NT x NT taps separate: the CTA first spreads the NT
 // lattice rows of the column's angle into a rho profile in shared memory,
 //   r[n] = sum_a B(theta_l - theta_{m0+a}) H[m0 + a][n],
-// for every time piece at once (shared memory: [np][nrho_max] profiles),
+// for every time piece at once (shared memory: [np][pstride] profiles),
 // then every output takes NT taps of each piece's profile and sums the
 // pieces in a fixed order. Outputs outside a piece's valid range skip its
 // table.
 template <int NT>
-__global__ void __launch_bounds__(256) k_interp_columns(const PieceDev* __restrict__ pieces,
-                                                        const int4* __restrict__ cmap, int nrho_max,
+__global__ void __launch_bounds__(256, NT == 4 ? 8 : 6) k_interp_columns(const PieceDev* __restrict__ pieces,
+                                                        const int4* __restrict__ cmap, int pstride,
                                                         int ntau_all, int np_all, float* __restrict__ g) {
     // np_all > 0: one gather with one slowness piece of np_all time pieces and
     // ntau_all outputs per column, column = block (no map load before the work)
     const int4 c = np_all > 0 ? make_int4(0, np_all, (int)blockIdx.x, 0) : __ldg(cmap + blockIdx.x);
     const int l = c.z, np = c.y;
     const int Ntau = np_all > 0 ? ntau_all : pieces[c.x].Ntau;
-    if (np > kMaxColPieces || (size_t)np * nrho_max * sizeof(float) > dyn_smem_bytes()) return;
+    if (np > kMaxColPieces || (size_t)np * pstride * sizeof(float) > dyn_smem_bytes()) return;
     // per-piece column data, loaded for all pieces at once
     __shared__ float4 s_w4[kMaxColPieces];
     __shared__ float2 s_w2[NT > 4 ? kMaxColPieces : 1];
@@ -1273,36 +517,49 @@ __global__ void __launch_bounds__(256) k_interp_columns(const PieceDev* __restri
     __shared__ const int2* s_rt[kMaxColPieces];
     __shared__ float s_sc[kMaxColPieces];
     __shared__ int2 s_rg[kMaxColPieces];
-    __shared__ int s_nr[kMaxColPieces];
+    __shared__ int s_nr[kMaxColPieces], s_lp[kMaxColPieces];
     if ((int)threadIdx.x < np) {
         const PieceDev& P = pieces[c.x + threadIdx.x];
         const int lc = l - P.l_lo;
         s_w4[threadIdx.x] = __ldg(P.colw + lc);
         if (NT > 4) s_w2[threadIdx.x] = __ldg(P.colw2 + lc);
         s_sc[threadIdx.x] = __ldg(P.colscale + lc);
-        s_r0[threadIdx.x] = P.lat + (size_t)__ldg(P.colm0 + lc) * P.Nrho;
+        s_r0[threadIdx.x] = P.lat + (size_t)__ldg(P.colm0 + lc) * P.lp;
+        s_lp[threadIdx.x] = P.lp;
         s_rt[threadIdx.x] = reinterpret_cast<const int2*>(P.rtab + (size_t)lc * Ntau);
         s_rg[threadIdx.x] = __ldg(P.rrange + lc);
         s_nr[threadIdx.x] = P.Nrho;
     }
     __syncthreads();
     // theta taps (the column's NT lattice rows) of every piece: the rho
-    // profiles, np * nrho_max floats; all pieces' loads in flight together
+    // profiles, np * pstride floats; four cells per thread and load (the
+    // lattice rows are 16-byte aligned), all pieces' loads in flight together
     for (int p = 0; p < np; ++p) {
-        const int Nr = s_nr[p];
+        const int Nr = s_nr[p], lp = s_lp[p];
         const float4 w4 = s_w4[p];
+        const float2 w2 = NT > 4 ? s_w2[p] : make_float2(0.f, 0.f);
         const float* r0 = s_r0[p];
-        float* prof = smem_f + p * nrho_max;
-#pragma unroll 2
-        for (int n = threadIdx.x; n < Nr; n += blockDim.x) {
-            const float a0 = __ldg(r0 + n), a1 = __ldg(r0 + Nr + n);
-            const float a2 = __ldg(r0 + 2 * Nr + n), a3 = __ldg(r0 + 3 * Nr + n);
-            if (NT > 4) {
-                const float2 w2 = s_w2[p];
-                const float a4 = __ldg(r0 + 4 * Nr + n), a5 = __ldg(r0 + 5 * Nr + n);
-                prof[n] = w4.x * a0 + w4.y * a1 + w4.z * a2 + w4.w * a3 + w2.x * a4 + w2.y * a5;
-            } else {
-                prof[n] = w4.x * a0 + w4.y * a1 + w4.z * a2 + w4.w * a3;
+        float* prof = smem_f + p * pstride;
+        for (int n = 4 * threadIdx.x; n < Nr; n += 4 * blockDim.x) {
+            float4 a[NT];
+#pragma unroll
+            for (int k = 0; k < NT; ++k) a[k] = __ldg(reinterpret_cast<const float4*>(r0 + (size_t)k * lp + n));
+            const float w[6] = {w4.x, w4.y, w4.z, w4.w, w2.x, w2.y};
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < NT; ++k) {
+                v.x = fmaf(w[k], a[k].x, v.x);
+                v.y = fmaf(w[k], a[k].y, v.y);
+                v.z = fmaf(w[k], a[k].z, v.z);
+                v.w = fmaf(w[k], a[k].w, v.w);
+            }
+            if (!(pstride & 3)) {
+                *reinterpret_cast<float4*>(prof + n) = v;
+            } else {                                   // profiles packed to fit shared memory
+                prof[n] = v.x;
+                if (n + 1 < Nr) prof[n + 1] = v.y;
+                if (n + 2 < Nr) prof[n + 2] = v.z;
+                if (n + 3 < Nr) prof[n + 3] = v.w;
             }
         }
     }
@@ -1326,7 +583,7 @@ __global__ void __launch_bounds__(256) k_interp_columns(const PieceDev* __restri
                 e[u] = (i >= rg.x && i <= rg.y) ? __ldg(s_rt[p] + i) : make_int2(-1, 0);
             }
             const float scp = s_sc[p];
-            const float* rp = smem_f + p * nrho_max;
+            const float* rp = smem_f + p * pstride;
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 if (e[u].x < 0) continue;
@@ -1375,7 +632,7 @@ __global__ void __launch_bounds__(kSampleBlock, NT == 4 ? 8 : 4) k_gather_sample
         float wt[NT], wr[NT];
         bspline_weights<NT>(__int_as_float(e.y), wt);
         bspline_weights<NT>(__int_as_float(e.z), wr);
-        acc += w * taps_nt<NT>(P.lat, P.Nrho, e.x >> 16, e.x & 0xffff, wt, wr);
+        acc += w * taps_nt<NT>(P.lat, P.lp, e.x >> 16, e.x & 0xffff, wt, wr);
     }
     f[(np_all > 0 ? 0 : pieces[m.x].f_off) + idx] = acc;
 }
@@ -1554,60 +811,11 @@ __global__ void __launch_bounds__(256) k_direct_adj(const float* __restrict__ g,
 // --------------------------------------------------------------------------
 // Launchers
 // --------------------------------------------------------------------------
-static int check_launch() {
-    cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? 0 : (int)e;
-}
-
-size_t scatter_smem_bytes(const PieceDev& P) { return rows_smem(P); }
-
-size_t colconv_smem_bytes(const PieceDev& P) { return colconv_smem(P); }
-
 int max_smem_optin() {
     int dev = 0, v = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     return v;
-}
-
-// Dynamic shared-memory limit of a kernel: raised only when a launch needs
-// more than the largest value already set on this device (the attribute call
-// costs host time on every launch otherwise).
-static int set_smem(const void* fn, size_t bytes) {
-    struct Entry { const void* fn; int dev; size_t bytes; };
-    static std::mutex mu;
-    static std::vector<Entry> set;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    std::lock_guard<std::mutex> lock(mu);
-    for (const Entry& e : set)
-        if (e.fn == fn && e.dev == dev && e.bytes >= bytes) return 0;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e != cudaSuccess) return (int)e;
-    for (Entry& en : set)
-        if (en.fn == fn && en.dev == dev) {
-            en.bytes = bytes;
-            return 0;
-        }
-    set.push_back(Entry{fn, dev, bytes});
-    return 0;
-}
-
-// Batch descriptor of n pieces with count(piece) blocks each; returns the
-// total number of blocks.
-template <class F>
-static int make_batch(const PieceDev* P, int n, PieceBatch& B, F&& count) {
-    B.n = n;
-    int total = 0;
-    for (int k = 0; k < kMaxBatch; ++k) {
-        B.first[k] = total;
-        if (k < n) {
-            B.p[k] = P[k];
-            total += count(P[k]);
-        }
-    }
-    B.first[kMaxBatch] = total;
-    return total;
 }
 
 // Kernels with B-spline taps exist for 4 (cubic) and 6 (quintic) taps per
@@ -1633,70 +841,6 @@ int launch_grid_tiles(const PieceDev* P, int n, const float* f, void* stream) {
     return check_launch();
 }
 
-static size_t max_over(const PieceDev* P, int n, size_t (*fn)(const PieceDev&)) {
-    size_t m = 0;
-    for (int k = 0; k < n; ++k) m = std::max(m, fn(P[k]));
-    return m;
-}
-
-size_t rows_smem_bytes(const PieceDev& P) { return scatter_smem_bytes(P); }
-
-// One stage over n <= kMaxBatch pieces (descriptors as a parameter) or over
-// a device-resident batch (descriptors and block map in device memory).
-template <class Src>
-static int set_and_launch(void (*kern)(Src), int nb, size_t sm, const Src& B, void* stream) {
-    if (int e = set_smem((const void*)kern, sm)) return e;
-    if (nb > 0) kern<<<nb, 512, sm, (cudaStream_t)stream>>>(B);
-    return check_launch();
-}
-
-int launch_rows_r2c(const PieceDev* P, int n, void* stream) {
-    PieceBatch B;
-    const int nb = make_batch(P, n, B, [](const PieceDev& q) { return q.nbands; });
-    return set_and_launch(k_rows_r2c<PieceBatch>, nb, max_over(P, n, rows_smem_bytes), B, stream);
-}
-
-int launch_band_rows(const PieceDev* P, int n, void* stream) {
-    PieceBatch B;
-    const int nb = make_batch(P, n, B, [](const PieceDev& q) { return q.nbands; });
-    const size_t sm = max_over(P, n, rows_smem_bytes);
-    if (P[0].ntaps == 6) return set_and_launch(k_band_rows<PieceBatch, 6>, nb, sm, B, stream);
-    if (P[0].ntaps == 4) return set_and_launch(k_band_rows<PieceBatch, 4>, nb, sm, B, stream);
-    return (int)cudaErrorInvalidValue;
-}
-
-bool colconv_all_x256(const PieceDev* P, int n) {
-    for (int k = 0; k < n; ++k)
-        if (!colconv_x256(P[k].fftT)) return false;
-    return true;
-}
-
-template <class Src>
-static int launch_colconv_as(const Src& B, int nb, size_t sm, bool x256, int adjoint, void* stream) {
-    if (x256) {
-        if (int e = set_smem((const void*)k_colconv<Src, kColThreads>, sm)) return e;
-        if (nb > 0) k_colconv<Src, kColThreads><<<nb, kColThreads, sm, (cudaStream_t)stream>>>(B, adjoint);
-    } else {
-        if (int e = set_smem((const void*)k_colconv<Src, kColThreadsGeneral>, sm)) return e;
-        if (nb > 0)
-            k_colconv<Src, kColThreadsGeneral><<<nb, kColThreadsGeneral, sm, (cudaStream_t)stream>>>(B, adjoint);
-    }
-    return check_launch();
-}
-
-int launch_colconv(const PieceDev* P, int n, int adjoint, void* stream) {
-    const size_t sm = max_over(P, n, colconv_smem_bytes);
-    PieceBatch B;
-    const int nb = make_batch(P, n, B, [](const PieceDev& q) { return q.nkb; });
-    return launch_colconv_as(B, nb, sm, colconv_all_x256(P, n), adjoint, stream);
-}
-
-int launch_rows_c2r(const PieceDev* P, int n, void* stream) {
-    PieceBatch B;
-    const int nb = make_batch(P, n, B, [](const PieceDev& q) { return q.nbands; });
-    return set_and_launch(k_rows_c2r<PieceBatch>, nb, max_over(P, n, rows_smem_bytes), B, stream);
-}
-
 int launch_grid_tiles_dev(const DevBatch& S, int nblocks, int ntaps, const void* f, int in_type, void* stream) {
     if (nblocks <= 0) return 0;
     HR_TAPS(ntaps, {
@@ -1707,24 +851,6 @@ int launch_grid_tiles_dev(const DevBatch& S, int nblocks, int ntaps, const void*
             k_grid_tiles<DevBatch, float, NT><<<nblocks, kUnitChunks, 0, (cudaStream_t)stream>>>(S, (const float*)f);
     });
     return check_launch();
-}
-
-int launch_rows_r2c_dev(const DevBatch& S, int nblocks, size_t smem, void* stream) {
-    return set_and_launch(k_rows_r2c<DevBatch>, nblocks, smem, S, stream);
-}
-
-int launch_band_rows_dev(const DevBatch& S, int nblocks, int ntaps, size_t smem, void* stream) {
-    if (ntaps == 6) return set_and_launch(k_band_rows<DevBatch, 6>, nblocks, smem, S, stream);
-    if (ntaps == 4) return set_and_launch(k_band_rows<DevBatch, 4>, nblocks, smem, S, stream);
-    return (int)cudaErrorInvalidValue;
-}
-
-int launch_colconv_dev(const DevBatch& S, int nblocks, size_t smem, bool x256, int adjoint, void* stream) {
-    return launch_colconv_as(S, nblocks, smem, x256, adjoint, stream);
-}
-
-int launch_rows_c2r_dev(const DevBatch& S, int nblocks, size_t smem, void* stream) {
-    return set_and_launch(k_rows_c2r<DevBatch>, nblocks, smem, S, stream);
 }
 
 // Dynamic shared memory the per-column profile kernels (the output
@@ -1760,13 +886,16 @@ int launch_col_profiles_cols(const PieceDev* pieces, const int4* cmap, int ncols
 }
 
 int launch_interp_columns(const PieceDev* pieces, const int4* cmap, int ncols, int nrho_max, int np_max,
-                          int ntau_all, int np_all, int ntaps, float* g, void* stream) {
+                          int ntau_all, int np_all, int ntaps, size_t limit, float* g, void* stream) {
     if (np_max > kMaxColPieces) return (int)cudaErrorInvalidValue;
-    const size_t sm = (size_t)np_max * nrho_max * sizeof(float);
+    // profiles on 16-byte boundaries where shared memory holds them so
+    const int up = (nrho_max + 3) & ~3;
+    const int pstride = (size_t)np_max * up * sizeof(float) <= limit ? up : nrho_max;
+    const size_t sm = (size_t)np_max * pstride * sizeof(float);
     HR_TAPS(ntaps, {
         if (int e = set_smem((const void*)k_interp_columns<NT>, sm)) return e;
         if (ncols > 0)
-            k_interp_columns<NT><<<ncols, 256, sm, (cudaStream_t)stream>>>(pieces, cmap, nrho_max, ntau_all, np_all, g);
+            k_interp_columns<NT><<<ncols, 256, sm, (cudaStream_t)stream>>>(pieces, cmap, pstride, ntau_all, np_all, g);
     });
     return check_launch();
 }

@@ -93,8 +93,10 @@ FftPlan make_dif_fft_plan(int n) {
         fp.rad[p] = R[p];
         fp.st[p] = S[p];
         fp.tw[p] = ofs;
+        while ((1 << fp.lst[p]) < S[p]) ++fp.lst[p];
         ofs += stage_table_len(S[p], R[p]);
     }
+    fp.ntw = ofs;
     return fp;
 }
 
@@ -305,19 +307,24 @@ struct HostPiece {
     int n_theta = 0, n_rho = 0, Ntheta = 0, Nrho = 0, Ptheta = 0, Prho = 0, k1max = 0, k2max = 0;
     double dtheta = 0, drho = 0, theta0 = 0, rho0 = 0, theta_m = 0;
     std::vector<int> jfirst;
-    int Rmax = 1;                                  // most rows per band shared memory allows
+    int max_pairs = 1;                             // most pairs of rows per band shared memory allows
     int max_tile_chunks = 0;                       // most gridding chunks of one tile
     int order = 3;                                 // B-spline degree
-    const int2* lband_R[kMaxBandRows + 1] = {};    // band column ranges for each rows-per-band
+    const int2* lband_R[kMaxBandRows + 1] = {};    // band column ranges for 2, 4, 6 rows per band
     PieceDev dev{};
 };
 
-// Rows per band of a piece: the band count and column ranges follow.
-static void set_rows(HostPiece& h, int R) {
-    h.dev.R = R;
-    h.dev.nbands = (h.Ntheta + R - 1) / R;
-    h.dev.lband = h.lband_R[R];
+// Rows per band of a piece, in pairs (an odd number is rounded up, or down
+// where `down`), bounded by what shared memory holds: the band count and
+// column ranges follow.
+static void set_rows(HostPiece& h, int R, bool down = false) {
+    h.dev.Re = 2 * std::max(1, std::min(down ? R / 2 : (R + 1) / 2, h.max_pairs));
+    h.dev.nbands = (h.Ntheta + h.dev.Re - 1) / h.dev.Re;
+    h.dev.lband = h.lband_R[h.dev.Re];
 }
+// Odd rows per band are rounded down where the bands of a launch (rows
+// lattice rows in all) would not give every SM two CTAs.
+static bool rows_down(int R, long rows) { return rows < 2L * 152 * ((R + 1) & ~1); }
 
 struct radon_plan_s {
     radon_desc d{};
@@ -331,12 +338,14 @@ struct radon_plan_s {
     float* lat_all = nullptr;                    // every piece's lattice, back to back
     size_t lat_bytes = 0;
     std::vector<PieceDev> host_devs;             // host copies of the descriptors (launch parameters)
+    std::vector<int> row_tpb;                    // row-kernel threads of each group of kMaxBatch pieces
     const int4* cmap = nullptr;                  // output columns: (first piece, count, l, 0)
     int ncols = 0;
     int col_pieces = 0;                          // largest count of cmap
     const int4* smap = nullptr;                  // sample blocks: (first piece, count, first sample, 0)
     int nsblocks = 0;
     int nrho_max = 0;
+    size_t interp_limit = 0;                     // shared memory of the output interpolation's profiles
     std::vector<void*> allocs;
     size_t bytes = 0;
     // per-stage timing
@@ -568,9 +577,9 @@ radon_status make_geometry(const radon_desc& d, const Grid& g, const TPiece& tp,
 
 // zeta_hat on the lattice's frequency grid (FP64 quadrature on the device),
 // divided twice by the B-spline symbol and normalised for the kernels' FFT
-// conventions; stored in the blocked layout [nkb][k1max+1][CB].
-radon_status kernel_spectrum(radon_plan_s* p, const HostPiece& h, int CB, int nkb,
-                             std::vector<cf>& Kout) {
+// conventions; stored in the blocked layout [nkb][k1max+2], two columns per
+// element, the last entry of every block zero (the frequencies beyond k1max).
+radon_status kernel_spectrum(radon_plan_s* p, const HostPiece& h, int nkb, std::vector<float4>& Kout) {
     const int n1 = h.k1max + 1, n2 = h.k2max + 1;
     const double dw1 = 1.0 / (h.Ptheta * h.dtheta), dw2 = 1.0 / (h.Prho * h.drho);
     const double lc_m = std::log(std::cos(h.theta_m));
@@ -629,15 +638,16 @@ radon_status kernel_spectrum(radon_plan_s* p, const HostPiece& h, int CB, int nk
     // Normalisation of the kernels' transforms: the row real FFT pair without
     // its 1/2 factors gives 2 Prho, the unnormalised column pair Ptheta.
     const double norm = 1.0 / (2.0 * h.Ptheta * h.Prho);
-    Kout.assign((size_t)nkb * n1 * CB, cf{0.f, 0.f});
+    Kout.assign((size_t)nkb * (n1 + 1), make_float4(0.f, 0.f, 0.f, 0.f));
     for (int k1 = 0; k1 < n1; ++k1) {
         const double s1 = bspline_symbol((double)k1 / h.Ptheta, h.order);
         for (int k2 = 0; k2 < n2; ++k2) {
             const double s2 = bspline_symbol((double)k2 / h.Prho, h.order);
             const double den = (s1 * s2) * (s1 * s2);
             const double zr = 2.0 * Zr[(size_t)k1 * n2 + k2], zi = 2.0 * Zi[(size_t)k1 * n2 + k2];
-            const int kb = k2 / CB, c = k2 % CB;
-            Kout[((size_t)kb * n1 + k1) * CB + c] = {(float)(zr / den * norm), (float)(zi / den * norm)};
+            float4& e = Kout[(size_t)(k2 / 2) * (n1 + 1) + k1];
+            (k2 & 1 ? e.y : e.x) = (float)(zr / den * norm);
+            (k2 & 1 ? e.w : e.z) = (float)(zi / den * norm);
         }
     }
     return RADON_OK;
@@ -777,23 +787,9 @@ radon_status build_piece_tables(radon_plan_s* p, HostPiece& h, const std::vector
         return fail(RADON_ERR_UNSUPPORTED,
                     "FFT length " + std::to_string(std::max(h.Prho / 2, h.Ptheta)) +
                         " above the FFT passes' limit (4096, 6144 = 3*2048 or 5120 = 5*1024)");
-    // rows per band: any value up to what shared memory allows gives the same
-    // results; the descriptor's choice, else 3 until the plan times them
-    // (the row kernels pad each row of their band by one complex element)
-    const int Rmax = (int)std::min<size_t>(kMaxBandRows, (size_t)smem_max / ((h.Prho + 2) * sizeof(float)));
-    if (Rmax < 1) return fail(RADON_ERR_UNSUPPORTED, "row FFT length too large for shared memory");
-    h.Rmax = Rmax;
-    const int R = std::min(Rmax, d.rows_per_band > 0 ? d.rows_per_band : 3);
-    const int CB = 2;   // spectrum columns per column block (the column kernel holds both)
-    // the column kernel holds the column block, its slice of K and the twiddle tables
-    const size_t col_smem = ((size_t)h.Ptheta + h.k1max + 1) * 2 * sizeof(cf) +
-                            (size_t)((fft_dif_tables(h.Ptheta, nullptr) + 2) & ~1) * sizeof(cf);
-    if (col_smem > (size_t)smem_max)
-        return fail(RADON_ERR_UNSUPPORTED, "column FFT length too large for shared memory");
-    P.R = R;
-    P.CB = CB;
-    P.nkb = (h.k2max + 1 + CB - 1) / CB;
-    P.nbands = (h.Ntheta + R - 1) / R;
+    P.nkb = (h.k2max + 2) / 2;
+    P.sp = (h.Ntheta + 7) & ~7;
+    P.lp = (h.Nrho + 3) & ~3;
     P.Nt = d.Nt;
     P.Nx = d.Nx;
     P.jt_lo = h.jt_lo;
@@ -803,7 +799,16 @@ radon_status build_piece_tables(radon_plan_s* p, HostPiece& h, const std::vector
     P.l_lo = h.l_lo;
     P.l_hi = h.l_hi;
     P.fftM = make_dif_fft_plan(h.Prho / 2);
+    // rows per band: any value up to what shared memory allows gives the same
+    // results; the descriptor's choice, else 3 until the plan times them
+    h.max_pairs = max_row_pairs(P, (size_t)smem_max);
+    if (h.max_pairs < 1) return fail(RADON_ERR_UNSUPPORTED, "row FFT length too large for shared memory");
     P.fftT = make_dif_fft_plan(h.Ptheta);
+    P.C = 1;
+    P.nkg = P.nkb;
+    // the column kernel holds a column block, its slice of K and a pass's twiddles
+    if (colconv_smem_bytes(P) > (size_t)smem_max)
+        return fail(RADON_ERR_UNSUPPORTED, "column FFT length too large for shared memory");
 
     // per-time weight (window, 2 a^2 tb, quadrature and B-spline normalisation)
     // and trapezoid weights in x, both FP64 for the position-table kernel
@@ -843,7 +848,7 @@ radon_status build_piece_tables(radon_plan_s* p, HostPiece& h, const std::vector
     }
     // candidate output columns of every band of rb rows: those whose NT
     // theta taps m0 .. m0+NT-1 meet the band
-    for (int rb = 1; rb <= Rmax; ++rb) {
+    for (int rb = 2; rb <= 2 * h.max_pairs; rb += 2) {
         const int nbands = (h.Ntheta + rb - 1) / rb;
         std::vector<int2> lband(nbands, int2{1, 0});
         for (int lc = 0; lc < ncol; ++lc) {
@@ -862,23 +867,29 @@ radon_status build_piece_tables(radon_plan_s* p, HostPiece& h, const std::vector
         }
         if (radon_status s = dev_upload(p, lband, &h.lband_R[rb])) return s;
     }
-    set_rows(h, R);
+    set_rows(h, d.rows_per_band > 0 ? d.rows_per_band : 3);
     // twiddles
     const int M = h.Prho / 2;
-    std::vector<cf> twM(fft_dif_tables(M, nullptr) + 1), twP(M + 1), twT((fft_dif_tables(h.Ptheta, nullptr) + 2) & ~1);
-    fft_dif_tables(M, twM.data());
-    fft_dif_tables(h.Ptheta, twT.data());
+    std::vector<cf> twP(M + 1);
+    // pass tables, every factor as a pair for the packed arithmetic
+    auto paired_tables = [](int n) {
+        std::vector<cf> w(fft_dif_tables(n, nullptr) + 1);
+        fft_dif_tables(n, w.data());
+        std::vector<float4> out;
+        for (const cf& v : w) out.push_back(make_float4(v.x, v.x, v.y, v.y));
+        return out;
+    };
+    const std::vector<float4> twM = paired_tables(M), twT = paired_tables(h.Ptheta);
     std::vector<int> rpos(M);
     {
         int R[kMaxDifPasses], S[kMaxDifPasses];
         const int s = dif_plan(M, R, S);
-        for (int k = 0; k < M; ++k) rpos[k] = dif_pos(s, R, S, k);
+        for (int k = 0; k < M; ++k) rpos[k] = dif_pos(s, R, S, k) + dif_pos(s, R, S, k) / 16;   // pad16
     }
-    P.twT_len = (int)twT.size();
     for (int k = 0; k <= M; ++k)
         twP[k] = {(float)std::cos(-2 * kPi * k / h.Prho), (float)std::sin(-2 * kPi * k / h.Prho)};
-    std::vector<cf> K;
-    if (radon_status s = kernel_spectrum(p, h, CB, P.nkb, K)) return s;
+    std::vector<float4> K;
+    if (radon_status s = kernel_spectrum(p, h, P.nkb, K)) return s;
 
     radon_status s = RADON_OK;
     if (NT > 4 && (s = dev_upload(p, colw2, &P.colw2))) return s;
@@ -965,10 +976,10 @@ size_t round256b(size_t v) { return (v + 255) & ~(size_t)255; }
 // The lattice of a piece followed by the arrival counters of its split
 // gridding tiles (cleared together before every forward gridding).
 size_t piece_lattice_bytes(const PieceDev& P) {
-    return round256b((size_t)P.Ntheta * P.Nrho * sizeof(float) + (size_t)P.ncount * sizeof(int));
+    return round256b((size_t)P.Ntheta * P.lp * sizeof(float) + (size_t)P.ncount * sizeof(int));
 }
 size_t piece_slot_bytes(const PieceDev& P) { return round256b((size_t)P.nslots * kTileRows * kTileCols * sizeof(float)); }
-size_t piece_spectrum_bytes(const PieceDev& P) { return round256b((size_t)P.nkb * P.CB * P.Ntheta * sizeof(cf)); }
+size_t piece_spectrum_bytes(const PieceDev& P) { return round256b((size_t)P.nkb * P.sp * sizeof(float4)); }
 size_t piece_profile_bytes(const PieceDev& P) {
     return round256b((size_t)(P.l_hi - P.l_lo + 1) * P.hpitch * sizeof(float));
 }
@@ -1160,7 +1171,7 @@ static int tune_rows(int rmax, Run&& run, void* stream) {
     }
     int best = 0;
     float best_ms = 0.f;
-    for (int R = 1; R <= rmax; ++R) {
+    for (int R = 2; R <= rmax; R += 2) {        // the rows go in pairs
         if (run(R) != 0) break;                     // warm-up (shared-memory attributes, caches)
         cudaEventRecord(a, (cudaStream_t)stream);
         for (int rep = 0; rep < 3; ++rep)
@@ -1178,6 +1189,13 @@ static int tune_rows(int rmax, Run&& run, void* stream) {
     cudaEventDestroy(b);
     cudaGetLastError();
     return best;
+}
+
+// Row-kernel threads of one launch over n pieces.
+static int plan_row_threads(const PieceDev* P, int n) {
+    size_t sm = 0;
+    for (int k = 0; k < n; ++k) sm = std::max(sm, rows_smem_bytes(P[k]));
+    return rows_threads(P, n, sm);
 }
 
 extern "C" radon_status radon_plan_create_ex(radon_plan* out, const radon_desc* din) {
@@ -1212,7 +1230,7 @@ extern "C" radon_status radon_plan_create_grid(radon_plan* out, const radon_desc
     void* const prof_base = prof;
     for (auto& h : p->pieces) {
         h.dev.lat = (float*)lat;
-        h.dev.spec = (cf*)spec;
+        h.dev.spec = (float4*)spec;
         h.dev.prof = (float*)prof;
         lat = (char*)lat + piece_lattice_bytes(h.dev);
         spec = (char*)spec + piece_spectrum_bytes(h.dev);
@@ -1220,7 +1238,7 @@ extern "C" radon_status radon_plan_create_grid(radon_plan* out, const radon_desc
     }
     if (p->d.rows_per_band == 0) {
         int rmax = kMaxBandRows;
-        for (auto& h : p->pieces) rmax = std::min(rmax, h.Rmax);
+        for (auto& h : p->pieces) rmax = std::min(rmax, 2 * h.max_pairs);
         cudaMemset(p->lat_all, 0, lat_b);
         cudaMemset(spec_base, 0, spec_b);
         cudaMemset(prof_base, 0, prof_b);
@@ -1235,9 +1253,10 @@ extern "C" radon_status radon_plan_create_grid(radon_plan* out, const radon_desc
                 }
                 for (int i = 0; i < np; i += kMaxBatch) {
                     const int n = std::min(kMaxBatch, np - i);
-                    if (int e = launch_rows_r2c(P.data() + i, n, nullptr)) return e;
-                    if (int e = launch_band_rows(P.data() + i, n, nullptr)) return e;
-                    if (int e = launch_rows_c2r(P.data() + i, n, nullptr)) return e;
+                    const int tpb = plan_row_threads(P.data() + i, n);
+                    if (int e = launch_rows_r2c(P.data() + i, n, tpb, nullptr)) return e;
+                    if (int e = launch_band_rows(P.data() + i, n, tpb, nullptr)) return e;
+                    if (int e = launch_rows_c2r(P.data() + i, n, tpb, nullptr)) return e;
                 }
                 return 0;
             },
@@ -1246,9 +1265,18 @@ extern "C" radon_status radon_plan_create_grid(radon_plan* out, const radon_desc
         for (auto& h : p->pieces) set_rows(h, R);
         p->d.rows_per_band = R;
     }
+    long rows = 0;
+    for (auto& h : p->pieces) rows += h.Ntheta;
     std::vector<PieceDev> devs;
-    for (auto& h : p->pieces) devs.push_back(h.dev);
+    for (auto& h : p->pieces) {
+        set_rows(h, p->d.rows_per_band, rows_down(p->d.rows_per_band, rows));
+        devs.push_back(h.dev);
+    }
+    set_col_groups(devs.data(), (int)devs.size());
+    for (size_t i = 0; i < devs.size(); ++i) p->pieces[i].dev = devs[i];
     p->host_devs = devs;
+    for (int i = 0; i < (int)devs.size(); i += kMaxBatch)
+        p->row_tpb.push_back(plan_row_threads(devs.data() + i, std::min(kMaxBatch, (int)devs.size() - i)));
     const PieceDev* dp = nullptr;
     if ((s = dev_upload(p, devs, &dp))) { destroy_plan(p); return s; }
     p->dev_pieces = const_cast<PieceDev*>(dp);
@@ -1264,7 +1292,8 @@ extern "C" radon_status radon_plan_create_grid(radon_plan* out, const radon_desc
     for (const int4& c : cmap) p->col_pieces = std::max(p->col_pieces, c.y);
     p->nsblocks = (int)smap.size();
     // the output interpolation holds one rho profile per time piece of a column
-    if ((size_t)p->col_pieces * p->nrho_max * sizeof(float) > interp_smem_limit(spline_taps(p->d.spline_order))) {
+    p->interp_limit = interp_smem_limit(spline_taps(p->d.spline_order));
+    if ((size_t)p->col_pieces * p->nrho_max * sizeof(float) > p->interp_limit) {
         destroy_plan(p);
         return fail(RADON_ERR_UNSUPPORTED, "too many time pieces for the lattice length along rho "
                                            "(the output interpolation's profiles exceed shared memory)");
@@ -1306,38 +1335,38 @@ static radon_status run_forward(radon_plan_s* p, const PieceDev* P, const PieceD
     }
     auto groups = [&](auto&& launch) {
         for (int i = 0; i < np; i += kMaxBatch)
-            if (int e = launch(P + i, std::min(kMaxBatch, np - i))) return e;
+            if (int e = launch(P + i, std::min(kMaxBatch, np - i), p->row_tpb[i / kMaxBatch])) return e;
         return 0;
     };
     if (radon_status s = cuda_status(
             timed(p, 0, b_samp + b_lat, stream,
                   [&] {
                       if (cudaError_t e = cudaMemsetAsync(lat, 0, lat_bytes, (cudaStream_t)stream)) return (int)e;
-                      return groups([&](const PieceDev* q, int n) { return launch_grid_tiles(q, n, f, stream); });
+                      return groups([&](const PieceDev* q, int n, int) { return launch_grid_tiles(q, n, f, stream); });
                   }),
             "gridding"))
         return s;
     if (radon_status s = cuda_status(
             timed(p, 1, b_lat + b_spec, stream,
-                  [&] { return groups([&](const PieceDev* q, int n) { return launch_rows_r2c(q, n, stream); }); }),
+                  [&] { return groups([&](const PieceDev* q, int n, int tpb) { return launch_rows_r2c(q, n, tpb, stream); }); }),
             "row FFT"))
         return s;
     if (radon_status s = cuda_status(
             timed(p, 2, 2 * b_spec + b_ker, stream,
-                  [&] { return groups([&](const PieceDev* q, int n) { return launch_colconv(q, n, 0, stream); }); }),
+                  [&] { return groups([&](const PieceDev* q, int n, int) { return launch_colconv(q, n, 0, stream); }); }),
             "convolution"))
         return s;
     if (radon_status s = cuda_status(
             timed(p, 3, b_spec + b_lat, stream,
-                  [&] { return groups([&](const PieceDev* q, int n) { return launch_rows_c2r(q, n, stream); }); }),
+                  [&] { return groups([&](const PieceDev* q, int n, int tpb) { return launch_rows_c2r(q, n, tpb, stream); }); }),
             "inverse row FFT"))
         return s;
     const double gb = 4.0 * p->d.Ntau * p->d.Nq;
     if (radon_status s = cuda_status(
             timed(p, 4, b_lat + gb, stream,
                   [&] { return launch_interp_columns(dP, p->cmap, p->ncols, p->nrho_max, p->col_pieces, p->d.Ntau,
-                                               p->qpieces.size() == 1 ? np : 0, spline_taps(p->d.spline_order), g,
-                                               stream); }),
+                                               p->qpieces.size() == 1 ? np : 0, spline_taps(p->d.spline_order),
+                                               p->interp_limit, g, stream); }),
             "interpolation"))
         return s;
     return RADON_OK;
@@ -1370,7 +1399,7 @@ extern "C" radon_status radon_adj(radon_plan p, const float* g, float* f, void* 
     }
     auto groups = [&](auto&& launch) {
         for (int i = 0; i < np; i += kMaxBatch)
-            if (int e = launch(P.data() + i, std::min(kMaxBatch, np - i))) return e;
+            if (int e = launch(P.data() + i, std::min(kMaxBatch, np - i), p->row_tpb[i / kMaxBatch])) return e;
         return 0;
     };
     if (radon_status s = cuda_status(
@@ -1384,17 +1413,17 @@ extern "C" radon_status radon_adj(radon_plan p, const float* g, float* f, void* 
         return s;
     if (radon_status s = cuda_status(
             timed(p, 5, b_h + b_spec, stream,
-                  [&] { return groups([&](const PieceDev* q, int n) { return launch_band_rows(q, n, stream); }); }),
+                  [&] { return groups([&](const PieceDev* q, int n, int tpb) { return launch_band_rows(q, n, tpb, stream); }); }),
             "adjoint interpolation (bands)"))
         return s;
     if (radon_status s = cuda_status(
             timed(p, 6, 2 * b_spec + b_ker, stream,
-                  [&] { return groups([&](const PieceDev* q, int n) { return launch_colconv(q, n, 1, stream); }); }),
+                  [&] { return groups([&](const PieceDev* q, int n, int) { return launch_colconv(q, n, 1, stream); }); }),
             "adjoint convolution"))
         return s;
     if (radon_status s = cuda_status(
             timed(p, 7, b_spec + b_lat, stream,
-                  [&] { return groups([&](const PieceDev* q, int n) { return launch_rows_c2r(q, n, stream); }); }),
+                  [&] { return groups([&](const PieceDev* q, int n, int tpb) { return launch_rows_c2r(q, n, tpb, stream); }); }),
             "inverse row FFT"))
         return s;
     return cuda_status(timed(p, 8, b_lat + 4.0 * p->d.Nt * p->d.Nx, stream,
@@ -1458,7 +1487,8 @@ extern "C" radon_status radon_plan_piece_lattice(radon_plan p, int piece, float*
         return fail(RADON_ERR_INVALID_ARG,
                     "out holds " + std::to_string(count) + " floats, the lattice has " + std::to_string(n));
     DeviceGuard guard(p->device);
-    if (cudaDeviceSynchronize() != cudaSuccess || cudaMemcpy(out, P.lat, n * sizeof(float), cudaMemcpyDeviceToHost) != cudaSuccess)
+    if (cudaDeviceSynchronize() != cudaSuccess || cudaMemcpy2D(out, P.Nrho * sizeof(float), P.lat, P.lp * sizeof(float), P.Nrho * sizeof(float), P.Ntheta,
+                     cudaMemcpyDeviceToHost) != cudaSuccess)
         return fail(RADON_ERR_CUDA, std::string("lattice copy failed: ") + cudaGetErrorString(cudaGetLastError()));
     return RADON_OK;
 }
@@ -1608,9 +1638,10 @@ struct radon_batch_s {
     const int4* smap = nullptr;
     int ncols = 0, nsblocks = 0, col_pieces = 0;
     size_t smem_rows = 0, smem_cols = 0;
+    int row_tpb = 128;                         // threads of the row kernels
     int nrho_max = 0;
+    size_t interp_limit = 0;                   // shared memory of the output interpolation's profiles
     int ntaps = 4;                             // B-spline taps per axis of every gather
-    bool col_x256 = false;                     // every piece takes the compile-time column pass
     float* lat_all = nullptr;
     size_t lat_bytes = 0;
 };
@@ -1701,6 +1732,7 @@ extern "C" radon_status radon_batch_create_grid(radon_batch* out, int n, const r
             P.g_off = b->g_off[i];
             host.push_back(P);
         }
+    set_col_groups(host.data(), (int)host.size());
     size_t lat_b = 0, spec_b = 0, prof_b = 0;
     for (auto& P : host) {
         lat_b += piece_lattice_bytes(P);
@@ -1720,7 +1752,7 @@ extern "C" radon_status radon_batch_create_grid(radon_batch* out, int n, const r
     void* const prof_base = prof;
     for (auto& P : host) {
         P.lat = (float*)lat;
-        P.spec = (cf*)spec;
+        P.spec = (float4*)spec;
         P.prof = (float*)prof;
         lat = (char*)lat + piece_lattice_bytes(P);
         spec = (char*)spec + piece_spectrum_bytes(P);
@@ -1729,14 +1761,14 @@ extern "C" radon_status radon_batch_create_grid(radon_batch* out, int n, const r
         b->smem_cols = std::max(b->smem_cols, colconv_smem_bytes(P));
         b->nrho_max = std::max(b->nrho_max, P.Nrho);
     }
-    b->col_x256 = colconv_all_x256(host.data(), (int)host.size());
+    b->row_tpb = rows_threads(host.data(), (int)host.size(), b->smem_rows);
     // block maps of the stage launches and the maps of the two gathers
     std::vector<int2> mu, mb, mk;
     for (int gi = 0; gi < (int)host.size(); ++gi) {
         const PieceDev& P = host[gi];
         for (int u = 0; u < P.nunits; ++u) mu.push_back(int2{gi, u});
         for (int u = 0; u < P.nbands; ++u) mb.push_back(int2{gi, u});
-        for (int u = 0; u < P.nkb; ++u) mk.push_back(int2{gi, u});
+        for (int u = 0; u < P.nkg; ++u) mk.push_back(int2{gi, u});
     }
     std::vector<int4> cmap, smap;
     int base = 0;
@@ -1758,7 +1790,8 @@ extern "C" radon_status radon_batch_create_grid(radon_batch* out, int n, const r
     b->ncols = (int)cmap.size();
     for (const int4& c : cmap) b->col_pieces = std::max(b->col_pieces, c.y);
     b->nsblocks = (int)smap.size();
-    if ((size_t)b->col_pieces * b->nrho_max * sizeof(float) > interp_smem_limit(b->ntaps)) {
+    b->interp_limit = interp_smem_limit(b->ntaps);
+    if ((size_t)b->col_pieces * b->nrho_max * sizeof(float) > b->interp_limit) {
         destroy_batch(b);
         return fail(RADON_ERR_UNSUPPORTED, "too many time pieces for the lattice length along rho "
                                            "(the output interpolation's profiles exceed shared memory)");
@@ -1768,7 +1801,7 @@ extern "C" radon_status radon_batch_create_grid(radon_batch* out, int n, const r
     int rmax = kMaxBandRows;
     for (int i = 0; i < n; ++i) tune = tune && descs[i].rows_per_band == 0;
     for (radon_plan_s* p : b->plans)
-        for (auto& h : p->pieces) rmax = std::min(rmax, h.Rmax);
+        for (auto& h : p->pieces) rmax = std::min(rmax, 2 * h.max_pairs);
     if (tune) {
         cudaMemset(b->lat_all, 0, b->lat_bytes);
         cudaMemset(spec_base, 0, spec_b);
@@ -1781,7 +1814,7 @@ extern "C" radon_status radon_batch_create_grid(radon_batch* out, int n, const r
             for (radon_plan_s* p : b->plans)
                 for (auto& h : p->pieces) {
                     set_rows(h, R);
-                    host[gi].R = h.dev.R;
+                    host[gi].Re = h.dev.Re;
                     host[gi].nbands = h.dev.nbands;
                     host[gi].lband = h.dev.lband;
                     // the row kernels' shared memory grows with R
@@ -1789,6 +1822,7 @@ extern "C" radon_status radon_batch_create_grid(radon_batch* out, int n, const r
                     for (int u = 0; u < host[gi].nbands; ++u) mb.push_back(int2{gi, u});
                     ++gi;
                 }
+            b->row_tpb = rows_threads(host.data(), (int)host.size(), b->smem_rows);
             radon_status st = RADON_OK;
             if ((st = dev_upload(b->store, host, &b->pieces)) || (st = dev_upload(b->store, mb, &b->map_bands)))
                 return st;
@@ -1801,17 +1835,18 @@ extern "C" radon_status radon_batch_create_grid(radon_batch* out, int n, const r
             [&](int R) {
                 if ((st = apply(R))) return 1;
                 const DevBatch Bd{b->pieces, b->map_bands};
-                if (int e = launch_rows_r2c_dev(Bd, b->n_bands, b->smem_rows, nullptr)) return e;
-                if (int e = launch_band_rows_dev(Bd, b->n_bands, b->ntaps, b->smem_rows, nullptr)) return e;
-                if (int e = launch_rows_c2r_dev(Bd, b->n_bands, b->smem_rows, nullptr)) return e;
+                if (int e = launch_rows_r2c_dev(Bd, b->n_bands, b->row_tpb, b->smem_rows, nullptr)) return e;
+                if (int e = launch_band_rows_dev(Bd, b->n_bands, b->ntaps, b->row_tpb, b->smem_rows, nullptr)) return e;
+                if (int e = launch_rows_c2r_dev(Bd, b->n_bands, b->row_tpb, b->smem_rows, nullptr)) return e;
                 return 0;
             },
             nullptr);
-        if (st || (st = apply(best > 0 ? best : std::min(3, rmax)))) {
+        const int R = best > 0 ? best : std::min(3, rmax);
+        if (st || (st = apply(R))) {
             destroy_batch(b);
             return st;
         }
-        for (radon_plan_s* p : b->plans) p->d.rows_per_band = host.empty() ? 3 : host[0].R;
+        for (radon_plan_s* p : b->plans) p->d.rows_per_band = R;
     }
     if (cudaDeviceSynchronize() != cudaSuccess) {
         destroy_batch(b);
@@ -1855,12 +1890,13 @@ extern "C" radon_status radon_batch_fwd(radon_batch b, const void* f, int in_typ
     if (cudaError_t e = cudaMemsetAsync(b->lat_all, 0, b->lat_bytes, (cudaStream_t)stream))
         return cuda_status((int)e, "clearing the lattices");
     if (radon_status s = cuda_status(launch_grid_tiles_dev(U, b->n_units, b->ntaps, f, in_type, stream), "gridding")) return s;
-    if (radon_status s = cuda_status(launch_rows_r2c_dev(Bd, b->n_bands, b->smem_rows, stream), "row FFT")) return s;
-    if (radon_status s = cuda_status(launch_colconv_dev(K, b->n_kb, b->smem_cols, b->col_x256, 0, stream), "convolution"))
+    if (radon_status s = cuda_status(launch_rows_r2c_dev(Bd, b->n_bands, b->row_tpb, b->smem_rows, stream), "row FFT")) return s;
+    if (radon_status s = cuda_status(launch_colconv_dev(K, b->n_kb, b->smem_cols, 0, stream), "convolution"))
         return s;
-    if (radon_status s = cuda_status(launch_rows_c2r_dev(Bd, b->n_bands, b->smem_rows, stream), "inverse row FFT"))
+    if (radon_status s = cuda_status(launch_rows_c2r_dev(Bd, b->n_bands, b->row_tpb, b->smem_rows, stream), "inverse row FFT"))
         return s;
-    return cuda_status(launch_interp_columns(b->pieces, b->cmap, b->ncols, b->nrho_max, b->col_pieces, 0, 0, b->ntaps, g, stream),
+    return cuda_status(launch_interp_columns(b->pieces, b->cmap, b->ncols, b->nrho_max, b->col_pieces, 0, 0, b->ntaps, b->interp_limit, g,
+                                             stream),
                        "interpolation");
 }
 
@@ -1873,12 +1909,12 @@ extern "C" radon_status radon_batch_adj(radon_batch b, const float* g, float* f,
                                                               0, 0, b->ntaps, g, stream),
                                      "adjoint interpolation (profiles)"))
         return s;
-    if (radon_status s = cuda_status(launch_band_rows_dev(Bd, b->n_bands, b->ntaps, b->smem_rows, stream),
+    if (radon_status s = cuda_status(launch_band_rows_dev(Bd, b->n_bands, b->ntaps, b->row_tpb, b->smem_rows, stream),
                                      "adjoint interpolation (bands)"))
         return s;
-    if (radon_status s = cuda_status(launch_colconv_dev(K, b->n_kb, b->smem_cols, b->col_x256, 1, stream), "adjoint convolution"))
+    if (radon_status s = cuda_status(launch_colconv_dev(K, b->n_kb, b->smem_cols, 1, stream), "adjoint convolution"))
         return s;
-    if (radon_status s = cuda_status(launch_rows_c2r_dev(Bd, b->n_bands, b->smem_rows, stream), "inverse row FFT"))
+    if (radon_status s = cuda_status(launch_rows_c2r_dev(Bd, b->n_bands, b->row_tpb, b->smem_rows, stream), "inverse row FFT"))
         return s;
     return cuda_status(launch_gather_samples(b->pieces, b->smap, b->nsblocks, f, 0, 0, 0, b->ntaps, stream), "adjoint gridding");
 }
@@ -1932,7 +1968,7 @@ int plan_forward_in_work(radon_plan_s* p, const float* f, float* g, void* work, 
         lat_bytes += piece_lattice_bytes(local[i]);
     }
     for (int i = 0; i < np; ++i) {
-        local[i].spec = (cf*)(base + off);
+        local[i].spec = (float4*)(base + off);
         off += piece_spectrum_bytes(local[i]);
     }
     for (int i = 0; i < np; ++i) {
