@@ -29,7 +29,14 @@ namespace hr {
 // so. The slices of K and the middle passes' twiddles are copied to shared
 // memory (cp.async) while pass 0 runs.
 // --------------------------------------------------------------------------
-constexpr int kColThreads = 160;   // radix-16 butterflies of a 2560-point column; 90 % of them busy at 2304
+// Threads of a CTA: 160, the radix-16 butterflies of a 2560-point column (90 %
+// busy at 2304; three CTAs per SM), or more, a butterfly each, for the longer
+// columns, of which shared memory holds only one or two per SM.
+constexpr int kColThreads = 160;
+constexpr int kColThreadsMax = 384;
+// 480 threads at 128 registers fill the register file: three CTAs of 160, two
+// of 192 to 224, one of 256 and more.
+constexpr int kColThreadsReg = 480;
 // 16-byte asynchronous copies global -> shared (cp.async; the completion
 // wait is the hardware's, no spin loop).
 __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
@@ -56,9 +63,9 @@ __host__ __device__ __forceinline__ size_t colconv_smem(const PieceDev& P) {
 // holds whenever the padding is as long as the lattice), so the butterfly
 // skips them, and the last pass the outputs there.
 template <int R, int LS, int NZ>
-__device__ __forceinline__ void col_first(c2* A, const c2* col, int sp, int Nth, int nc, int lsr, const c2* T, int t) {
+__device__ __forceinline__ void col_first(c2* A, const c2* col, int sp, int Nth, int nc, int lsr, const c2* T, int t, int nt) {
     const int ls = LS ? LS : lsr, S = 1 << ls, SP = first_step(ls);
-    for (int i = t; i < nc << ls; i += kColThreads) {
+    for (int i = t; i < nc << ls; i += nt) {
         const int cp = i >> ls, m = i & (S - 1);
         const c2* src = col + (size_t)cp * sp + m;
         c2 x[R];
@@ -78,9 +85,9 @@ __device__ __forceinline__ void col_first(c2* A, const c2* col, int sp, int Nth,
 }
 // Inverse pass 0, shared to global memory.
 template <int R, int LS, int NZ>
-__device__ __forceinline__ void col_last(const c2* A, c2* col, int sp, int Nth, int nc, int lsr, const c2* T, int t) {
+__device__ __forceinline__ void col_last(const c2* A, c2* col, int sp, int Nth, int nc, int lsr, const c2* T, int t, int nt) {
     const int ls = LS ? LS : lsr, S = 1 << ls, SP = first_step(ls);
-    for (int i = t; i < nc << ls; i += kColThreads) {
+    for (int i = t; i < nc << ls; i += nt) {
         const int cp = i >> ls, m = i & (S - 1);
         const c2* Z = A + cp * (SP * R) + pad16(m);
         c2 x[R];
@@ -96,18 +103,18 @@ __device__ __forceinline__ void col_last(const c2* A, c2* col, int sp, int Nth, 
     }
 }
 template <int R>
-__device__ __forceinline__ void col_first_any(c2* A, const c2* col, int sp, int Nth, int nc, int ls, const c2* T, int t) {
+__device__ __forceinline__ void col_first_any(c2* A, const c2* col, int sp, int Nth, int nc, int ls, const c2* T, int t, int nt) {
     constexpr int H = (R + 1) / 2;
-    if (Nth > H << ls) col_first<R, 0, R>(A, col, sp, Nth, nc, ls, T, t);
-    else if (R >= 5 && ls == 8) col_first<R, R >= 5 ? 8 : 0, H>(A, col, sp, Nth, nc, ls, T, t);
-    else col_first<R, 0, H>(A, col, sp, Nth, nc, ls, T, t);
+    if (Nth > H << ls) col_first<R, 0, R>(A, col, sp, Nth, nc, ls, T, t, nt);
+    else if (R >= 5 && ls == 8) col_first<R, R >= 5 ? 8 : 0, H>(A, col, sp, Nth, nc, ls, T, t, nt);
+    else col_first<R, 0, H>(A, col, sp, Nth, nc, ls, T, t, nt);
 }
 template <int R>
-__device__ __forceinline__ void col_last_any(const c2* A, c2* col, int sp, int Nth, int nc, int ls, const c2* T, int t) {
+__device__ __forceinline__ void col_last_any(const c2* A, c2* col, int sp, int Nth, int nc, int ls, const c2* T, int t, int nt) {
     constexpr int H = (R + 1) / 2;
-    if (Nth > H << ls) col_last<R, 0, R>(A, col, sp, Nth, nc, ls, T, t);
-    else if (R >= 5 && ls == 8) col_last<R, R >= 5 ? 8 : 0, H>(A, col, sp, Nth, nc, ls, T, t);
-    else col_last<R, 0, H>(A, col, sp, Nth, nc, ls, T, t);
+    if (Nth > H << ls) col_last<R, 0, R>(A, col, sp, Nth, nc, ls, T, t, nt);
+    else if (R >= 5 && ls == 8) col_last<R, R >= 5 ? 8 : 0, H>(A, col, sp, Nth, nc, ls, T, t, nt);
+    else col_last<R, 0, H>(A, col, sp, Nth, nc, ls, T, t, nt);
 }
 
 // x K or x conj(K), exchanged.
@@ -202,9 +209,9 @@ __device__ __forceinline__ void col_middle16(c2* A, const FftPlan& fp, const c2*
 
 // The last pass of a plan of any length.
 template <int R, bool ADJ>
-__device__ __forceinline__ void col_kernel_any(c2* A, const FftPlan& fp, const c2* K, int k1n, int nc, int t) {
+__device__ __forceinline__ void col_kernel_any(c2* A, const FftPlan& fp, const c2* K, int k1n, int nc, int t, int nt) {
     const int n = fp.n, s = fp.nst, nb = n / R, pitch = seq_pitch(n, fp.rad[0]);
-    for (int i = t; i < nc * nb; i += kColThreads) {
+    for (int i = t; i < nc * nb; i += nt) {
         const int cp = i / nb, b = i - cp * nb;
         int fb = 0, w = 1, rem = b;
         for (int p = 0; p + 1 < s; ++p) {
@@ -237,7 +244,7 @@ __device__ __forceinline__ void col_kernel_any(c2* A, const FftPlan& fp, const c
     default: CALL(2); break;
 
 template <class Src, bool ADJ>
-__global__ void __launch_bounds__(kColThreads, 3) k_colconv(const __grid_constant__ Src B) {
+__global__ void __launch_bounds__(kColThreadsReg, 1) k_colconv(const __grid_constant__ Src B) {
     int bx;
     const PieceDev& P = piece_of(B, bx);
     const int n = P.Ptheta, Nth = P.Ntheta, k1n = P.k1max + 2, sp = P.sp;   // K ends with a zero
@@ -245,7 +252,7 @@ __global__ void __launch_bounds__(kColThreads, 3) k_colconv(const __grid_constan
     const int kb0 = bx * P.C, nc = min(P.C, P.nkb - kb0);
     const int pitch = seq_pitch(n, P.fftT.rad[0]);
     const FftPlan& fp = P.fftT;
-    const int s = fp.nst, ntw = col_twiddles(fp), t = threadIdx.x;
+    const int s = fp.nst, ntw = col_twiddles(fp), t = threadIdx.x, nt = blockDim.x;
     c2* A = reinterpret_cast<c2*>(smem_f);
     c2* K = A + P.C * pitch;
     c2* Ts = K + P.C * k1n;
@@ -253,54 +260,54 @@ __global__ void __launch_bounds__(kColThreads, 3) k_colconv(const __grid_constan
     const c2* Tg = reinterpret_cast<const c2*>(P.twT);
     {
         const c2* Kg = reinterpret_cast<const c2*>(P.K) + (size_t)kb0 * k1n;
-        for (int i = t; i < nc * k1n; i += kColThreads) cp_async16(K + i, Kg + i);
+        for (int i = t; i < nc * k1n; i += nt) cp_async16(K + i, Kg + i);
         const c2* Tm = Tg + (ntw ? fp.tw[1] : 0);
-        for (int i = t; i < ntw; i += kColThreads) cp_async16(Ts + i, Tm + i);
+        for (int i = t; i < ntw; i += nt) cp_async16(Ts + i, Tm + i);
     }
     if (!fft_by16(n)) {
-        for (int i = t; i < nc * Nth; i += kColThreads) {
+        for (int i = t; i < nc * Nth; i += nt) {
             const int cp = i / Nth, m = i - cp * Nth;
             const ulonglong2 v = __ldcg(reinterpret_cast<const ulonglong2*>(col + (size_t)cp * sp + m));
             st2(A + cp * pitch + pad16(m), c2{v.x, v.y});
         }
-        for (int i = t; i < nc * (n - Nth); i += kColThreads) {
+        for (int i = t; i < nc * (n - Nth); i += nt) {
             const int cp = i / (n - Nth), m = Nth + i - cp * (n - Nth);
             st2(A + cp * pitch + pad16(m), c2{0ull, 0ull});
         }
         cp_async_wait_all();
         __syncthreads();
         for (int p = 0; p + 1 < s; ++p) {
-#define HR_CF(RR) pass_any<RR, false>(A, pitch, nc, n / RR, fp.st[p], Tg + fp.tw[p], t, kColThreads)
+#define HR_CF(RR) pass_any<RR, false>(A, pitch, nc, n / RR, fp.st[p], Tg + fp.tw[p], t, nt)
             switch (fp.rad[p]) { HR_RADIX_CASES(HR_CF) }
             __syncthreads();
         }
-#define HR_K(RR) col_kernel_any<RR, ADJ>(A, fp, K, k1n, nc, t)
+#define HR_K(RR) col_kernel_any<RR, ADJ>(A, fp, K, k1n, nc, t, nt)
         switch (fp.rad[s - 1]) { HR_RADIX_CASES(HR_K) }
         __syncthreads();
         for (int p = s - 2; p >= 0; --p) {
-#define HR_CI(RR) pass_any<RR, true>(A, pitch, nc, n / RR, fp.st[p], Tg + fp.tw[p], t, kColThreads)
+#define HR_CI(RR) pass_any<RR, true>(A, pitch, nc, n / RR, fp.st[p], Tg + fp.tw[p], t, nt)
             switch (fp.rad[p]) { HR_RADIX_CASES(HR_CI) }
             __syncthreads();
         }
-        for (int i = t; i < nc * Nth; i += kColThreads) {
+        for (int i = t; i < nc * Nth; i += nt) {
             const int cp = i / Nth, m = i - cp * Nth;
             st2(col + (size_t)cp * sp + m, ld2(A + cp * pitch + pad16(m)));
         }
         return;
     }
     const int ls0 = fp.lst[0];
-#define HR_FIRST(RR) col_first_any<RR>(A, col, sp, Nth, nc, ls0, Tg, t)
+#define HR_FIRST(RR) col_first_any<RR>(A, col, sp, Nth, nc, ls0, Tg, t, nt)
     switch (fp.rad[0]) { HR_RADIX_CASES(HR_FIRST) }
     cp_async_wait_all();
     __syncthreads();
     const int nall = nc * n;                       // elements of the CTA's blocks, back to back
     if (s == 4) {
-        pass16<4, false>(A, t, nall >> 2, kColThreads, fp.lst[1], ls0, Ts);
+        pass16<4, false>(A, t, nall >> 2, nt, fp.lst[1], ls0, Ts);
         __syncthreads();
     }
     const int r1 = s >= 3 ? fp.rad[s - 2] : 0;
     const c2* T1 = Ts + (s >= 3 ? fp.tw[s - 2] - fp.tw[1] : 0);
-    const Team w(nall, t, kColThreads);
+    const Team w(nall, t, nt);
     for (int e0 = w.first; e0 < nall; e0 += w.next) {
         const int b = (e0 >> 4) + w.me;
         const bool on = 16 * b < nall;
@@ -322,10 +329,10 @@ __global__ void __launch_bounds__(kColThreads, 3) k_colconv(const __grid_constan
     }
     __syncthreads();
     if (s == 4) {
-        pass16<4, true>(A, t, nall >> 2, kColThreads, fp.lst[1], ls0, Ts);
+        pass16<4, true>(A, t, nall >> 2, nt, fp.lst[1], ls0, Ts);
         __syncthreads();
     }
-#define HR_LAST(RR) col_last_any<RR>(A, col, sp, Nth, nc, ls0, Tg, t)
+#define HR_LAST(RR) col_last_any<RR>(A, col, sp, Nth, nc, ls0, Tg, t, nt)
     switch (fp.rad[0]) { HR_RADIX_CASES(HR_LAST) }
 }
 
@@ -344,10 +351,16 @@ void set_col_groups(PieceDev* P, int n) {
     }
 }
 
+int col_threads(const PieceDev* P, int n) {
+    int t = kColThreads;
+    for (int k = 0; k < n; ++k) t = std::max(t, std::min(kColThreadsMax, (P[k].Ptheta / 16 * P[k].C + 31) & ~31));
+    return t;
+}
+
 template <class Src, bool ADJ>
-static int launch_colconv_as(const Src& B, int nb, size_t sm, void* stream) {
+static int launch_colconv_as(const Src& B, int nb, int tpb, size_t sm, void* stream) {
     if (int e = set_smem((const void*)k_colconv<Src, ADJ>, sm)) return e;
-    if (nb > 0) k_colconv<Src, ADJ><<<nb, kColThreads, sm, (cudaStream_t)stream>>>(B);
+    if (nb > 0) k_colconv<Src, ADJ><<<nb, tpb, sm, (cudaStream_t)stream>>>(B);
     return check_launch();
 }
 
@@ -355,14 +368,14 @@ int launch_colconv(const PieceDev* P, int n, int adjoint, void* stream) {
     size_t sm = 0;
     for (int k = 0; k < n; ++k) sm = std::max(sm, colconv_smem(P[k]));
     PieceBatch B;
-    const int nb = make_batch(P, n, B, [](const PieceDev& q) { return q.nkg; });
-    return adjoint ? launch_colconv_as<PieceBatch, true>(B, nb, sm, stream)
-                   : launch_colconv_as<PieceBatch, false>(B, nb, sm, stream);
+    const int nb = make_batch(P, n, B, [](const PieceDev& q) { return q.nkg; }), tpb = col_threads(P, n);
+    return adjoint ? launch_colconv_as<PieceBatch, true>(B, nb, tpb, sm, stream)
+                   : launch_colconv_as<PieceBatch, false>(B, nb, tpb, sm, stream);
 }
 
-int launch_colconv_dev(const DevBatch& S, int nblocks, size_t smem, int adjoint, void* stream) {
-    return adjoint ? launch_colconv_as<DevBatch, true>(S, nblocks, smem, stream)
-                   : launch_colconv_as<DevBatch, false>(S, nblocks, smem, stream);
+int launch_colconv_dev(const DevBatch& S, int nblocks, int tpb, size_t smem, int adjoint, void* stream) {
+    return adjoint ? launch_colconv_as<DevBatch, true>(S, nblocks, tpb, smem, stream)
+                   : launch_colconv_as<DevBatch, false>(S, nblocks, tpb, smem, stream);
 }
 
 }  // namespace hr

@@ -149,7 +149,9 @@ int max_row_pairs(const PieceDev& P, size_t smem_max);
 int launch_grid_tiles_dev(const DevBatch& S, int nblocks, int ntaps, const void* f, int in_type, void* stream);
 int launch_rows_r2c_dev(const DevBatch& S, int nblocks, int tpb, size_t smem, void* stream);
 int launch_band_rows_dev(const DevBatch& S, int nblocks, int ntaps, int tpb, size_t smem, void* stream);
-int launch_colconv_dev(const DevBatch& S, int nblocks, size_t smem, int adjoint, void* stream);
+int launch_colconv_dev(const DevBatch& S, int nblocks, int tpb, size_t smem, int adjoint, void* stream);
+// Threads of a column-pass CTA for one launch over the n pieces.
+int col_threads(const PieceDev* P, int n);
 // Column blocks per CTA (C, nkg) of every piece of one launch: as many as
 // give the CTA's threads a butterfly each, but no fewer than two CTAs per SM
 // (304) over the launch, so that a small gather still spreads over the chip.

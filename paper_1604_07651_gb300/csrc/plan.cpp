@@ -1638,7 +1638,7 @@ struct radon_batch_s {
     const int4* smap = nullptr;
     int ncols = 0, nsblocks = 0, col_pieces = 0;
     size_t smem_rows = 0, smem_cols = 0;
-    int row_tpb = 128;                         // threads of the row kernels
+    int row_tpb = 128, col_tpb = 160;          // threads of the row and column kernels
     int nrho_max = 0;
     size_t interp_limit = 0;                   // shared memory of the output interpolation's profiles
     int ntaps = 4;                             // B-spline taps per axis of every gather
@@ -1762,6 +1762,7 @@ extern "C" radon_status radon_batch_create_grid(radon_batch* out, int n, const r
         b->nrho_max = std::max(b->nrho_max, P.Nrho);
     }
     b->row_tpb = rows_threads(host.data(), (int)host.size(), b->smem_rows);
+    b->col_tpb = col_threads(host.data(), (int)host.size());
     // block maps of the stage launches and the maps of the two gathers
     std::vector<int2> mu, mb, mk;
     for (int gi = 0; gi < (int)host.size(); ++gi) {
@@ -1891,7 +1892,7 @@ extern "C" radon_status radon_batch_fwd(radon_batch b, const void* f, int in_typ
         return cuda_status((int)e, "clearing the lattices");
     if (radon_status s = cuda_status(launch_grid_tiles_dev(U, b->n_units, b->ntaps, f, in_type, stream), "gridding")) return s;
     if (radon_status s = cuda_status(launch_rows_r2c_dev(Bd, b->n_bands, b->row_tpb, b->smem_rows, stream), "row FFT")) return s;
-    if (radon_status s = cuda_status(launch_colconv_dev(K, b->n_kb, b->smem_cols, 0, stream), "convolution"))
+    if (radon_status s = cuda_status(launch_colconv_dev(K, b->n_kb, b->col_tpb, b->smem_cols, 0, stream), "convolution"))
         return s;
     if (radon_status s = cuda_status(launch_rows_c2r_dev(Bd, b->n_bands, b->row_tpb, b->smem_rows, stream), "inverse row FFT"))
         return s;
@@ -1912,7 +1913,7 @@ extern "C" radon_status radon_batch_adj(radon_batch b, const float* g, float* f,
     if (radon_status s = cuda_status(launch_band_rows_dev(Bd, b->n_bands, b->ntaps, b->row_tpb, b->smem_rows, stream),
                                      "adjoint interpolation (bands)"))
         return s;
-    if (radon_status s = cuda_status(launch_colconv_dev(K, b->n_kb, b->smem_cols, 1, stream), "adjoint convolution"))
+    if (radon_status s = cuda_status(launch_colconv_dev(K, b->n_kb, b->col_tpb, b->smem_cols, 1, stream), "adjoint convolution"))
         return s;
     if (radon_status s = cuda_status(launch_rows_c2r_dev(Bd, b->n_bands, b->row_tpb, b->smem_rows, stream), "inverse row FFT"))
         return s;
