@@ -170,11 +170,15 @@ int launch_interp_columns(const PieceDev* pieces, const int4* cmap, int ncols, i
 // per output column (cmap / np_all / shared memory as the interpolation's).
 int launch_col_profiles_cols(const PieceDev* pieces, const int4* cmap, int ncols, int nrho_max, int np_max,
                              int ntau_all, int np_all, int ntaps, const float* g, void* stream);
-// Adjoint gather: one CTA per kSampleBlock samples of one gather;
-// smap[b] = (first piece, number of pieces, first sample, 0), or, when
-// np_all > 0 (one gather of Nt_all x Nx_all samples in np_all pieces),
-// samples [b kSampleBlock, (b + 1) kSampleBlock).
+// Adjoint gather: CTAs of kSampleBlock samples of one gather, 32 per 16 times
+// of two traces, in order along the traces; smap[b] = (first piece, number of
+// pieces, block, 0), or, when np_all > 0 (one gather of Nt_all x Nx_all samples
+// in np_all pieces), block b.
 constexpr int kSampleBlock = 256;
+inline int sample_blocks(int Nt, int Nx) {
+    const long warps = (long)((Nt + 15) / 16) * ((Nx + 1) / 2);
+    return (int)((warps * 32 + kSampleBlock - 1) / kSampleBlock);
+}
 int launch_gather_samples(const PieceDev* pieces, const int4* smap, int nblocks, float* f, int np_all, int Nt_all,
                           int Nx_all, int ntaps, void* stream);
 size_t rows_smem_bytes(const PieceDev& P);

@@ -606,22 +606,27 @@ __global__ void __launch_bounds__(256, NT == 4 ? 8 : 6) k_interp_columns(const P
 
 // Adjoint of the gridding (transpose of Eq. (15)): every gather sample reads
 // the NT x NT taps of each sub-problem that holds it. One CTA per kSampleBlock
-// samples of one gather: smap[b] = (first piece, number of pieces, first
-// sample of the block within the gather).
+// sample slots of one gather, a warp 16 times of two neighbouring traces
+// (sample_blocks): smap[b] = (first piece, number of pieces, block within the
+// gather). Bound: the L1 request rate. A tap load of a warp
+// touches 3 to 4.5 lines at 2048^2 so, against 3.4 to 7 with 32 times of one
+// trace (a curve through the lattice crosses rows); 8 x 4 touches as many
+// there, but more where traces are sparse.
 template <int NT>
 __global__ void __launch_bounds__(kSampleBlock, NT == 4 ? 8 : 4) k_gather_samples(const PieceDev* __restrict__ pieces,
                                                                     const int4* __restrict__ smap,
                                                                     float* __restrict__ f, int np_all, int Nt_all,
                                                                     int Nx_all) {
     // np_all > 0: one gather of Nt_all x Nx_all samples in np_all pieces,
-    // samples = blocks in order (no map load before the work)
-    const int4 m = np_all > 0 ? make_int4(0, np_all, (int)blockIdx.x * kSampleBlock, 0) : __ldg(smap + blockIdx.x);
+    // its blocks in order (no map load before the work)
+    const int4 m = np_all > 0 ? make_int4(0, np_all, (int)blockIdx.x, 0) : __ldg(smap + blockIdx.x);
     const int Nt = np_all > 0 ? Nt_all : pieces[m.x].Nt;
     const int Nx = np_all > 0 ? Nx_all : pieces[m.x].Nx;
-    const long idx = (long)m.z + threadIdx.x;
-    if (idx >= (long)Nt * Nx) return;
-    const int k = (int)(idx / Nt);
-    const int j = (int)(idx - (long)k * Nt);
+    const unsigned wp = (unsigned)m.z * (kSampleBlock / 32) + (threadIdx.x >> 5), per = (unsigned)((Nt + 15) >> 4);
+    const int kp = (int)(wp / per);
+    const int j = (int)(wp - (unsigned)kp * per) * 16 + (threadIdx.x & 15), k = 2 * kp + (threadIdx.x >> 4 & 1);
+    if (j >= Nt || k >= Nx) return;
+    const long idx = (long)k * Nt + j;
     float acc = 0.f;
     for (int p = m.x; p < m.x + m.y; ++p) {
         const PieceDev& P = pieces[p];

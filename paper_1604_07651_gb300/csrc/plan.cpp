@@ -342,7 +342,7 @@ struct radon_plan_s {
     const int4* cmap = nullptr;                  // output columns: (first piece, count, l, 0)
     int ncols = 0;
     int col_pieces = 0;                          // largest count of cmap
-    const int4* smap = nullptr;                  // sample blocks: (first piece, count, first sample, 0)
+    const int4* smap = nullptr;                  // sample blocks: (first piece, count, block, 0)
     int nsblocks = 0;
     int nrho_max = 0;
     size_t interp_limit = 0;                     // shared memory of the output interpolation's profiles
@@ -995,9 +995,8 @@ void column_map(const radon_plan_s* p, int base, std::vector<int4>& out) {
 
 // Sample blocks of a plan's gather for the adjoint gather kernel.
 void sample_map(const radon_plan_s* p, int base, int, std::vector<int4>& out) {
-    const long n = (long)p->d.Nt * p->d.Nx;
-    for (long b = 0; b < n; b += kSampleBlock)
-        out.push_back(int4{base, (int)p->pieces.size(), (int)b, 0});
+    const int n = sample_blocks(p->d.Nt, p->d.Nx);
+    for (int b = 0; b < n; ++b) out.push_back(int4{base, (int)p->pieces.size(), b, 0});
 }
 
 void destroy_plan(radon_plan_s* p) {
