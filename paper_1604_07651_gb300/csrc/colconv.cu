@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(kColThreadsReg, 1) k_colconv(const __grid_cons
     int bx;
     const PieceDev& P = piece_of(B, bx);
     const int n = P.Ptheta, Nth = P.Ntheta, k1n = P.k1max + 2, sp = P.sp;   // K ends with a zero
-    if (colconv_smem(P) > dyn_smem_bytes()) return;
+    if (colconv_smem(P) > dyn_smem_bytes()) return chain_wait<5>();
     const int kb0 = bx * P.C, nc = min(P.C, P.nkb - kb0);
     const int pitch = seq_pitch(n, P.fftT.rad[0]);
     const FftPlan& fp = P.fftT;
@@ -264,6 +264,8 @@ __global__ void __launch_bounds__(kColThreadsReg, 1) k_colconv(const __grid_cons
         const c2* Tm = Tg + (ntw ? fp.tw[1] : 0);
         for (int i = t; i < ntw; i += nt) cp_async16(Ts + i, Tm + i);
     }
+    chain_next<5>();
+    chain_wait<5>();
     if (!fft_by16(n)) {
         for (int i = t; i < nc * Nth; i += nt) {
             const int cp = i / Nth, m = i - cp * Nth;
@@ -360,8 +362,7 @@ int col_threads(const PieceDev* P, int n) {
 template <class Src, bool ADJ>
 static int launch_colconv_as(const Src& B, int nb, int tpb, size_t sm, void* stream) {
     if (int e = set_smem((const void*)k_colconv<Src, ADJ>, sm)) return e;
-    if (nb > 0) k_colconv<Src, ADJ><<<nb, tpb, sm, (cudaStream_t)stream>>>(B);
-    return check_launch();
+    return nb > 0 ? launch_chain(5, k_colconv<Src, ADJ>, nb, tpb, sm, stream, B) : 0;
 }
 
 int launch_colconv(const PieceDev* P, int n, int adjoint, void* stream) {

@@ -27,13 +27,20 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "device.cuh"
 
 namespace hr {
 
-__device__ __forceinline__ float load_in(const float* p) { return __ldg(p); }
-__device__ __forceinline__ float load_in(const __nv_bfloat16* p) { return __bfloat162float(__ldg(p)); }
+// Data another kernel of the stream writes (gathers, images, lattices,
+// profiles) are read with ordinary global loads (__ldca): with dependent
+// launches the read-only path (__ldg, __restrict__) is for the plan's tables
+// alone.
+__device__ __forceinline__ float load_in(const float* p) { return __ldca(p); }
+__device__ __forceinline__ float load_in(const __nv_bfloat16* p) {
+    return __int_as_float((unsigned)__ldca(reinterpret_cast<const unsigned short*>(p)) << 16);
+}
 
 // Shared gridding tile: the kTileRows x kTileCols cells plus a halo of
 // NT - 1 cells on every side (NT taps per axis: 4 cubic, 6 quintic), so that
@@ -95,7 +102,11 @@ __device__ __forceinline__ float block_max_abs(float v, float* red) {
 }
 
 // Forward gridding (Eq. (15)) of the gather f[Nx][Nt] onto the lattice
-// P.lat (zeroed before). The plan lists, per tile of kTileRows x kTileCols
+// P.lat. Every cell is written, a tile without samples has an empty unit (one
+// launch less than clearing first: 2 of 40 us at 256 x 64); a batch's lattices
+// are cleared before, which is the faster way where the units have no time to
+// spare (128 gathers: 2074 against 2109 us).
+// The plan lists, per tile of kTileRows x kTileCols
 // cells, chunks of at most 8 consecutive samples of one trace whose NT x NT
 // footprint meets the tile, and cuts every tile's list into work units of at
 // most kUnitChunks chunks (sample density varies by two orders of magnitude
@@ -214,7 +225,7 @@ __device__ __forceinline__ void grid_merge_split(const PieceDev& P, int4 us, int
 
 template <class Src, class T, int NT>
 __global__ void __launch_bounds__(kUnitChunks, NT == 4 ? 4 : 2) k_grid_tiles(const __grid_constant__ Src B,
-                                                                             const T* __restrict__ f) {
+                                                                             const T* f) {
     using Tile = GridTile<NT>;
     __shared__ int tile[Tile::rows * Tile::pitch];
     __shared__ float red[kUnitChunks / 32];
@@ -223,6 +234,19 @@ __global__ void __launch_bounds__(kUnitChunks, NT == 4 ? 4 : 2) k_grid_tiles(con
     const int4 u = __ldg(P.units + bx);           // (tile, first chunk, end chunk, 28 - ec)
     const int ti = u.x / P.ntc, tj = u.x - ti * P.ntc;
     const int m_lo = ti * kTileRows, n_lo = tj * kTileCols;
+    const int nr = min(kTileRows, P.Ntheta - m_lo), nc = min(kTileCols, P.Nrho - n_lo);
+    chain_next<8>();
+    constexpr bool kCleared = std::is_same<Src, DevBatch>::value;   // a batch's lattices are cleared before
+    if (kCleared) chain_wait<8>();                // (after the clearing, nothing to start early for)
+    if (u.y == u.z) {                             // a tile without samples
+        if (kCleared) return;
+        chain_wait<8>();
+        for (int i = threadIdx.x; i < kTileRows * kTileCols; i += blockDim.x) {
+            const int m = i / kTileCols, n = i - m * kTileCols;
+            if (m < nr && n < nc) P.lat[(size_t)(m_lo + m) * P.lp + n_lo + n] = 0.f;
+        }
+        return;
+    }
     for (int i = threadIdx.x; i < Tile::rows * Tile::pitch; i += blockDim.x) tile[i] = 0;
     // one chunk per thread: issue every load of the chunk before the first is used
     const int c = u.y + threadIdx.x;
@@ -236,13 +260,13 @@ __global__ void __launch_bounds__(kUnitChunks, NT == 4 ? 4 : 2) k_grid_tiles(con
         const T* fk = f + P.f_off + (size_t)ch.x * P.Nt + ch.y;
 #pragma unroll
         for (int s = 0; s < 8; ++s) {
-            if (s < ch.z) {
-                ent[s] = __ldg(st + s);
-                v[s] = load_in(fk + s);
-            } else {
-                ent[s] = make_int4(0, 0, 0, 0);
-                v[s] = 0.f;
-            }
+            ent[s] = s < ch.z ? __ldg(st + s) : make_int4(0, 0, 0, 0);
+            if (kCleared) v[s] = s < ch.z ? load_in(fk + s) : 0.f;
+        }
+        if (!kCleared) {
+            chain_wait<8>();
+#pragma unroll
+            for (int s = 0; s < 8; ++s) v[s] = s < ch.z ? load_in(fk + s) : 0.f;
         }
 #pragma unroll
         for (int s = 0; s < 8; ++s) {
@@ -254,12 +278,11 @@ __global__ void __launch_bounds__(kUnitChunks, NT == 4 ? 4 : 2) k_grid_tiles(con
     }
     vmax = block_max_abs(vmax, red);   // also orders the tile's zeroing before the adds
     const int4 us = __ldg(P.uslot + bx);  // (first slot, units of the tile, index, counter)
-    const int nr = min(kTileRows, P.Ntheta - m_lo), nc = min(kTileCols, P.Nrho - n_lo);
     if (!(vmax > 0.f && vmax <= 3.402823466e38f)) {   // all zero (nothing to add) or not finite (NaN tile)
         const float fill = vmax == 0.f ? 0.f : __int_as_float(0x7fc00000);
         if (us.y > 1) {
             grid_merge_split(P, us, m_lo, n_lo, nr, nc, [&](int) { return fill; });
-        } else if (fill != 0.f) {
+        } else if (fill != 0.f || !kCleared) {
             for (int i = threadIdx.x; i < kTileRows * kTileCols; i += blockDim.x) {
                 const int m = i / kTileCols, n = i - m * kTileCols;
                 if (m < nr && n < nc) P.lat[(size_t)(m_lo + m) * P.lp + n_lo + n] = fill;
@@ -319,7 +342,7 @@ __global__ void __launch_bounds__(kUnitChunks, NT == 4 ? 4 : 2) k_grid_tiles(con
     for (int i = threadIdx.x; i < kTileRows * kTileCols; i += blockDim.x) {   // the tile's only unit
         const int m = i / kTileCols, n = i - m * kTileCols;
         const int t = tile[(m + Tile::halo) * Tile::pitch + n + Tile::halo];
-        if (t != 0 && m < nr && n < nc) P.lat[(size_t)(m_lo + m) * P.lp + n_lo + n] = sc.down(t);
+        if ((t != 0 || !kCleared) && m < nr && n < nc) P.lat[(size_t)(m_lo + m) * P.lp + n_lo + n] = sc.down(t);
     }
 }
 
@@ -345,7 +368,9 @@ __global__ void __launch_bounds__(kUnitChunks, NT == 4 ? 4 : 2) k_grid_tiles(con
 template <int NT>
 __global__ void __launch_bounds__(256) k_col_profiles_cols(const PieceDev* __restrict__ pieces,
                                                            const int4* __restrict__ cmap, int nrho_max, int ntau_all,
-                                                           int np_all, const float* __restrict__ g) {
+                                                           int np_all, const float* g) {
+    chain_next<5>();
+    chain_wait<5>();
     const int4 c = np_all > 0 ? make_int4(0, np_all, (int)blockIdx.x, 0) : __ldg(cmap + blockIdx.x);
     const int l = c.z, np = c.y;
     const int Ntau = np_all > 0 ? ntau_all : pieces[c.x].Ntau;
@@ -379,7 +404,7 @@ __global__ void __launch_bounds__(256) k_col_profiles_cols(const PieceDev* __res
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
             const int i = i0 + q * (int)blockDim.x + threadIdx.x;
-            v[q] = i < Ntau ? __ldg(gl + i) : 0.f;
+            v[q] = i < Ntau ? __ldca(gl + i) : 0.f;
         }
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
@@ -410,7 +435,7 @@ __global__ void __launch_bounds__(256) k_col_profiles_cols(const PieceDev* __res
         const int ib = i0 + Q * (int)threadIdx.x;
         float v[Q];
 #pragma unroll
-        for (int q = 0; q < Q; ++q) v[q] = (ib + q >= lo && ib + q <= hi) ? __ldg(gl + ib + q) : 0.f;
+        for (int q = 0; q < Q; ++q) v[q] = (ib + q >= lo && ib + q <= hi) ? __ldca(gl + ib + q) : 0.f;
         for (int p = 0; p < np; ++p) {
             const int2 rg = s_rg[p];
             const int2* rt = s_rt[p];
@@ -476,15 +501,15 @@ __global__ void __launch_bounds__(256) k_col_profiles_cols(const PieceDev* __res
 
 // NT x NT taps of the lattice at first tap (m0, n0).
 template <int NT>
-__device__ __forceinline__ float taps_nt(const float* __restrict__ lat, int Nr, int m0, int n0,
+__device__ __forceinline__ float taps_nt(const float* lat, int Nr, int m0, int n0,
                                          const float (&wt)[NT], const float (&wr)[NT]) {
     float s = 0.f;
 #pragma unroll
     for (int a = 0; a < NT; ++a) {
         const float* row = lat + (size_t)(m0 + a) * Nr + n0;
-        float r = __ldg(row) * wr[0];
+        float r = __ldca(row) * wr[0];
 #pragma unroll
-        for (int c = 1; c < NT; ++c) r += __ldg(row + c) * wr[c];
+        for (int c = 1; c < NT; ++c) r += __ldca(row + c) * wr[c];
         s += wt[a] * r;
     }
     return s;
@@ -503,9 +528,11 @@ __device__ __forceinline__ float taps_nt(const float* __restrict__ lat, int Nr, 
 template <int NT>
 __global__ void __launch_bounds__(256, NT == 4 ? 8 : 6) k_interp_columns(const PieceDev* __restrict__ pieces,
                                                         const int4* __restrict__ cmap, int pstride,
-                                                        int ntau_all, int np_all, float* __restrict__ g) {
+                                                        int ntau_all, int np_all, float* g) {
     // np_all > 0: one gather with one slowness piece of np_all time pieces and
     // ntau_all outputs per column, column = block (no map load before the work)
+    chain_next<8>();
+    chain_wait<8>();
     const int4 c = np_all > 0 ? make_int4(0, np_all, (int)blockIdx.x, 0) : __ldg(cmap + blockIdx.x);
     const int l = c.z, np = c.y;
     const int Ntau = np_all > 0 ? ntau_all : pieces[c.x].Ntau;
@@ -543,7 +570,7 @@ __global__ void __launch_bounds__(256, NT == 4 ? 8 : 6) k_interp_columns(const P
         for (int n = 4 * threadIdx.x; n < Nr; n += 4 * blockDim.x) {
             float4 a[NT];
 #pragma unroll
-            for (int k = 0; k < NT; ++k) a[k] = __ldg(reinterpret_cast<const float4*>(r0 + (size_t)k * lp + n));
+            for (int k = 0; k < NT; ++k) a[k] = __ldca(reinterpret_cast<const float4*>(r0 + (size_t)k * lp + n));
             const float w[6] = {w4.x, w4.y, w4.z, w4.w, w2.x, w2.y};
             float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
@@ -615,10 +642,12 @@ __global__ void __launch_bounds__(256, NT == 4 ? 8 : 6) k_interp_columns(const P
 template <int NT>
 __global__ void __launch_bounds__(kSampleBlock, NT == 4 ? 8 : 4) k_gather_samples(const PieceDev* __restrict__ pieces,
                                                                     const int4* __restrict__ smap,
-                                                                    float* __restrict__ f, int np_all, int Nt_all,
+                                                                    float* f, int np_all, int Nt_all,
                                                                     int Nx_all) {
     // np_all > 0: one gather of Nt_all x Nx_all samples in np_all pieces,
     // its blocks in order (no map load before the work)
+    chain_next<8>();
+    chain_wait<8>();
     const int4 m = np_all > 0 ? make_int4(0, np_all, (int)blockIdx.x, 0) : __ldg(smap + blockIdx.x);
     const int Nt = np_all > 0 ? Nt_all : pieces[m.x].Nt;
     const int Nx = np_all > 0 ? Nx_all : pieces[m.x].Nx;
@@ -841,21 +870,19 @@ int max_smem_optin() {
 int launch_grid_tiles(const PieceDev* P, int n, const float* f, void* stream) {
     PieceBatch B;
     const int nb = make_batch(P, n, B, [](const PieceDev& q) { return q.nunits; });
-    if (nb > 0)
-        HR_TAPS(P[0].ntaps, (k_grid_tiles<PieceBatch, float, NT><<<nb, kUnitChunks, 0, (cudaStream_t)stream>>>(B, f)));
-    return check_launch();
+    if (nb > 0) HR_TAPS(P[0].ntaps, return launch_chain(8, k_grid_tiles<PieceBatch, float, NT>, nb, kUnitChunks, 0, stream, B, f));
+    return 0;
 }
 
 int launch_grid_tiles_dev(const DevBatch& S, int nblocks, int ntaps, const void* f, int in_type, void* stream) {
     if (nblocks <= 0) return 0;
     HR_TAPS(ntaps, {
         if (in_type == kInBF16)
-            k_grid_tiles<DevBatch, __nv_bfloat16, NT><<<nblocks, kUnitChunks, 0, (cudaStream_t)stream>>>(
-                S, (const __nv_bfloat16*)f);
-        else
-            k_grid_tiles<DevBatch, float, NT><<<nblocks, kUnitChunks, 0, (cudaStream_t)stream>>>(S, (const float*)f);
+            return launch_chain(8, k_grid_tiles<DevBatch, __nv_bfloat16, NT>, nblocks, kUnitChunks, 0, stream, S,
+                                (const __nv_bfloat16*)f);
+        return launch_chain(8, k_grid_tiles<DevBatch, float, NT>, nblocks, kUnitChunks, 0, stream, S, (const float*)f);
     });
-    return check_launch();
+    return 0;
 }
 
 // Dynamic shared memory the per-column profile kernels (the output
@@ -884,10 +911,9 @@ int launch_col_profiles_cols(const PieceDev* pieces, const int4* cmap, int ncols
     HR_TAPS(ntaps, {
         if (int e = set_smem((const void*)k_col_profiles_cols<NT>, sm)) return e;
         if (ncols > 0)
-            k_col_profiles_cols<NT><<<ncols, 256, sm, (cudaStream_t)stream>>>(pieces, cmap, nrho_max, ntau_all, np_all,
-                                                                              g);
+            return launch_chain(5, k_col_profiles_cols<NT>, ncols, 256, sm, stream, pieces, cmap, nrho_max, ntau_all, np_all, g);
     });
-    return check_launch();
+    return 0;
 }
 
 int launch_interp_columns(const PieceDev* pieces, const int4* cmap, int ncols, int nrho_max, int np_max,
@@ -900,17 +926,17 @@ int launch_interp_columns(const PieceDev* pieces, const int4* cmap, int ncols, i
     HR_TAPS(ntaps, {
         if (int e = set_smem((const void*)k_interp_columns<NT>, sm)) return e;
         if (ncols > 0)
-            k_interp_columns<NT><<<ncols, 256, sm, (cudaStream_t)stream>>>(pieces, cmap, pstride, ntau_all, np_all, g);
+            return launch_chain(8, k_interp_columns<NT>, ncols, 256, sm, stream, pieces, cmap, pstride, ntau_all, np_all, g);
     });
-    return check_launch();
+    return 0;
 }
 
 int launch_gather_samples(const PieceDev* pieces, const int4* smap, int nblocks, float* f, int np_all, int Nt_all,
                           int Nx_all, int ntaps, void* stream) {
     if (nblocks > 0)
-        HR_TAPS(ntaps, (k_gather_samples<NT><<<nblocks, kSampleBlock, 0, (cudaStream_t)stream>>>(pieces, smap, f, np_all,
-                                                                                                Nt_all, Nx_all)));
-    return check_launch();
+        HR_TAPS(ntaps, return launch_chain(8, k_gather_samples<NT>, nblocks, kSampleBlock, 0, stream, pieces, smap, f, np_all,
+                                           Nt_all, Nx_all));
+    return 0;
 }
 
 int launch_sample_table(const TableArgs& A, const double* cj, const double* wk, const int* jfirst,

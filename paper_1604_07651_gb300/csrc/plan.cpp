@@ -699,6 +699,10 @@ radon_status build_tile_lists(radon_plan_s* p, HostPiece& h, PieceDev& P) {
         const int base = (int)flat.size();
         const int m_lo = (t / P.ntc) * TR, n_lo = (t % P.ntc) * TC;
         flat.insert(flat.end(), runs[t].begin(), runs[t].end());
+        if (runs[t].empty()) {          // an empty unit: the tile's cells still have to be written
+            units.push_back(int4{t, base, base, 28});
+            uwork.push_back(0);
+        }
         for (int c = 0; c < (int)runs[t].size(); c += kUnitChunks) {
             const int e = std::min((int)runs[t].size(), c + kUnitChunks);
             long w = 0;
@@ -1235,10 +1239,13 @@ extern "C" radon_status radon_plan_create_grid(radon_plan* out, const radon_desc
         spec = (char*)spec + piece_spectrum_bytes(h.dev);
         prof = (char*)prof + piece_profile_bytes(h.dev);
     }
+    if (cudaMemset(p->lat_all, 0, lat_b) != cudaSuccess) {      // the gridding's counters start at zero
+        destroy_plan(p);
+        return fail(RADON_ERR_CUDA, "clearing the plan's buffers failed");
+    }
     if (p->d.rows_per_band == 0) {
         int rmax = kMaxBandRows;
         for (auto& h : p->pieces) rmax = std::min(rmax, 2 * h.max_pairs);
-        cudaMemset(p->lat_all, 0, lat_b);
         cudaMemset(spec_base, 0, spec_b);
         cudaMemset(prof_base, 0, prof_b);
         const int np = (int)p->pieces.size();
@@ -1319,11 +1326,11 @@ static radon_status cuda_status(int e, const char* what) {
 }
 
 // The forward chain over the pieces `P` (host copies; `dP` the same on the
-// device), lattices in [lat, lat + lat_bytes). Every stage is one launch per
+// device); the counters behind the lattices are zero between calls. Every stage is one launch per
 // group of at most kMaxBatch pieces; the output interpolation is one launch
 // over every output column.
-static radon_status run_forward(radon_plan_s* p, const PieceDev* P, const PieceDev* dP, float* lat,
-                                size_t lat_bytes, const float* f, float* g, void* stream) {
+static radon_status run_forward(radon_plan_s* p, const PieceDev* P, const PieceDev* dP, const float* f, float* g,
+                                void* stream) {
     const int np = (int)p->pieces.size();
     double b_samp = 0, b_lat = 0, b_spec = 0, b_ker = 0;
     for (int i = 0; i < np; ++i) {
@@ -1339,10 +1346,7 @@ static radon_status run_forward(radon_plan_s* p, const PieceDev* P, const PieceD
     };
     if (radon_status s = cuda_status(
             timed(p, 0, b_samp + b_lat, stream,
-                  [&] {
-                      if (cudaError_t e = cudaMemsetAsync(lat, 0, lat_bytes, (cudaStream_t)stream)) return (int)e;
-                      return groups([&](const PieceDev* q, int n, int) { return launch_grid_tiles(q, n, f, stream); });
-                  }),
+                  [&] { return groups([&](const PieceDev* q, int n, int) { return launch_grid_tiles(q, n, f, stream); }); }),
             "gridding"))
         return s;
     if (radon_status s = cuda_status(
@@ -1378,7 +1382,7 @@ extern "C" radon_status radon_fwd(radon_plan p, const float* f, float* g, void* 
     if (!f || !g) return fail(RADON_ERR_INVALID_ARG, "NULL data pointer");
     DeviceGuard guard(p->device);
     const std::vector<PieceDev>& P = host_pieces(p);
-    return run_forward(p, P.data(), p->dev_pieces, p->lat_all, p->lat_bytes, f, g, stream);
+    return run_forward(p, P.data(), p->dev_pieces, f, g, stream);
 }
 
 extern "C" radon_status radon_adj(radon_plan p, const float* g, float* f, void* stream) {
@@ -1978,7 +1982,9 @@ int plan_forward_in_work(radon_plan_s* p, const float* f, float* g, void* work, 
     DeviceGuard guard(p->device);
     if (radon_status s = cuda_status(launch_write_pieces(local, np, dpieces, stream), "piece descriptors"))
         return s;
-    return run_forward(p, local, dpieces, lat, lat_bytes, f, g, stream);
+    if (cudaError_t e = cudaMemsetAsync(lat, 0, lat_bytes, (cudaStream_t)stream))   // the gridding's counters
+        return cuda_status((int)e, "clearing the work area");
+    return run_forward(p, local, dpieces, f, g, stream);
 }
 
 }  // namespace hr

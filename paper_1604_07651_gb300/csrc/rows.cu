@@ -26,7 +26,7 @@ __host__ __device__ __forceinline__ size_t rows_smem(const PieceDev& P) {
 // lp, nrows of them exist) from global memory. NZ: the inputs from NZ on are
 // zero padding and not read.
 template <int R, int NZ>
-__device__ __forceinline__ void row_first(c2* A, const float* __restrict__ lat, int lp, int Nr, int nrows, int np, int ls,
+__device__ __forceinline__ void row_first(c2* A, const float* lat, int lp, int Nr, int nrows, int np, int ls,
                                           const c2* __restrict__ T, int t, int nt) {
     const int S = 1 << ls, SP = first_step(ls);
 #pragma unroll 2
@@ -40,8 +40,8 @@ __device__ __forceinline__ void row_first(c2* A, const float* __restrict__ lat, 
             const int n2 = 2 * (m + r * S);
             float2 a = make_float2(0.f, 0.f), b = a;
             if (n2 < Nr) {
-                a = __ldg(reinterpret_cast<const float2*>(s0 + 2 * r * S));
-                b = __ldg(reinterpret_cast<const float2*>(s1 + 2 * r * S));
+                a = __ldca(reinterpret_cast<const float2*>(s0 + 2 * r * S));
+                b = __ldca(reinterpret_cast<const float2*>(s1 + 2 * r * S));
                 if (n2 + 1 == Nr) a.y = b.y = 0.f;       // the pitch's padding
             }
             x[r] = {pk(a.x, b.x), pk(a.y, b.y)};
@@ -225,15 +225,15 @@ __device__ __forceinline__ void rows_pre(const PieceDev& P, c2* A, int pitch, in
             a0[u] = a1[u] = b0[u][0] = b0[u][1] = b1[u][0] = b1[u][1] = zero;
             if (i >= total) continue;
             if (2 * kb < nk) {
-                a0[u] = __ldg(row + (size_t)kb * P.sp);
-                a1[u] = __ldg(row + (size_t)kb * P.sp + 1);
+                a0[u] = __ldca(row + (size_t)kb * P.sp);
+                a1[u] = __ldca(row + (size_t)kb * P.sp + 1);
             }
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
                 const int k2 = M - 2 * kb - c;
                 if (k2 >= 0 && k2 < nk) {
-                    b0[u][c] = __ldg(row + (size_t)(k2 >> 1) * P.sp);
-                    b1[u][c] = __ldg(row + (size_t)(k2 >> 1) * P.sp + 1);
+                    b0[u][c] = __ldca(row + (size_t)(k2 >> 1) * P.sp);
+                    b1[u][c] = __ldca(row + (size_t)(k2 >> 1) * P.sp + 1);
                 }
             }
         }
@@ -270,6 +270,8 @@ template <class Src>
 __global__ void __launch_bounds__(kRowThreadsMax, 2) k_rows_r2c(const __grid_constant__ Src B) {
     int bx;
     const PieceDev& P = piece_of(B, bx);
+    chain_next<4>();
+    chain_wait<4>();
     if (rows_smem(P) > dyn_smem_bytes()) return;
     const int mb = bx * P.Re, nrows = min(P.Re, P.Ntheta - mb), np = (nrows + 1) / 2;
     const int M = P.Prho / 2, pitch = seq_pitch(M, P.fftM.rad[0]), t = threadIdx.x, nt = blockDim.x;
@@ -289,7 +291,7 @@ __global__ void __launch_bounds__(kRowThreadsMax, 2) k_rows_r2c(const __grid_con
             const int pr = i / M, n = i - pr * M;
             const float* s0 = lat + (size_t)(2 * pr) * P.lp;
             const float* s1 = 2 * pr + 1 < nrows ? s0 + P.lp : s0;
-            auto at = [&](const float* s, int j) { return j < P.Nrho ? __ldg(s + j) : 0.f; };
+            auto at = [&](const float* s, int j) { return j < P.Nrho ? __ldca(s + j) : 0.f; };
             st2(A + pr * pitch + pad16(n), c2{pk(at(s0, 2 * n), at(s1, 2 * n)), pk(at(s0, 2 * n + 1), at(s1, 2 * n + 1))});
         }
         __syncthreads();
@@ -304,6 +306,8 @@ template <class Src>
 __global__ void __launch_bounds__(kRowThreadsMax, 2) k_rows_c2r(const __grid_constant__ Src B) {
     int bx;
     const PieceDev& P = piece_of(B, bx);
+    chain_next<4>();
+    chain_wait<4>();
     if (rows_smem(P) > dyn_smem_bytes()) return;
     const int mb = bx * P.Re, nrows = min(P.Re, P.Ntheta - mb), np = (nrows + 1) / 2;
     const int M = P.Prho / 2, pitch = seq_pitch(M, P.fftM.rad[0]), t = threadIdx.x, nt = blockDim.x;
@@ -351,7 +355,7 @@ __device__ __forceinline__ void band_spread(const PieceDev& P, c2* A, int pitch,
                                             int t, int nt) {
     const int hp = P.hpitch, M = P.Prho / 2;
     const int ls0 = fft_by16(M) ? P.fftM.lst[0] : 30;            // 30: pass_any's layout
-    const float* __restrict__ h = P.prof;
+    const float* h = P.prof;
     const int ncol = max(0, lr.y - lr.x + 1);
     for (int n0 = 0; 2 * n0 < nz; n0 += nt) {
         const int n4 = n0 + t;
@@ -378,7 +382,7 @@ __device__ __forceinline__ void band_spread(const PieceDev& P, c2* A, int pitch,
                 const float* hl = h + (size_t)(lr.x + l0 - P.l_lo) * hp + 4 * n4;
 #pragma unroll 4
                 for (int c = 0; c < nl; ++c) {
-                    const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2*>(hl + (size_t)c * hp));
+                    const ulonglong2 v = __ldca(reinterpret_cast<const ulonglong2*>(hl + (size_t)c * hp));
 #pragma unroll
                     for (int r = 0; r < 2 * NP; ++r) {
                         acc[r][0] = fma2(wt[c][r], v.x, acc[r][0]);
@@ -432,6 +436,8 @@ __global__ void __launch_bounds__(kRowThreadsMax, 2) k_band_rows(const __grid_co
     __shared__ f2 wt[kBandCols * kMaxBandRows];
     int band;
     const PieceDev& P = piece_of(B, band);
+    chain_next<4>();
+    chain_wait<4>();
     if (rows_smem(P) > dyn_smem_bytes()) return;
     const int mb = band * P.Re, npb = P.Re / 2, np = (min(P.Re, P.Ntheta - mb) + 1) / 2;
     const int M = P.Prho / 2, pitch = seq_pitch(M, P.fftM.rad[0]), t = threadIdx.x, nt = blockDim.x;
@@ -503,8 +509,7 @@ int rows_threads(const PieceDev* P, int n, size_t smem) {
 template <class Src>
 static int set_and_launch(void (*kern)(Src), int nb, int tpb, size_t sm, const Src& B, void* stream) {
     if (int e = set_smem((const void*)kern, sm)) return e;
-    if (nb > 0) kern<<<nb, tpb, sm, (cudaStream_t)stream>>>(B);
-    return check_launch();
+    return nb > 0 ? launch_chain(4, kern, nb, tpb, sm, stream, B) : 0;
 }
 static size_t rows_smem_max(const PieceDev* P, int n) {
     size_t m = 0;

@@ -26,7 +26,7 @@
 #include <string>
 
 #include "hradon.h"
-#include "internal.h"
+#include "device.cuh"
 
 namespace hr {
 namespace {
@@ -35,20 +35,24 @@ constexpr int kThreads = 256;
 constexpr int kNormBlocks = 512;   // partial sums of the norm reduction
 
 // r = f - mask[k] * a  (a = R_h* y), over [Nx][Nt]; mask NULL means all ones.
-__global__ void __launch_bounds__(kThreads) k_residual(const float* __restrict__ f, const float* __restrict__ mask,
-                                                      float* __restrict__ r, int Nt, long n) {
+__global__ void __launch_bounds__(kThreads) k_residual(const float* f, const float* mask,
+                                                      float* r, int Nt, long n) {
+    chain_next<8>();
+    chain_wait<8>();
     for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-        const float m = mask ? __ldg(mask + i / Nt) : 1.f;
-        r[i] = __ldg(f + i) - m * r[i];
+        const float m = mask ? mask[i / Nt] : 1.f;
+        r[i] = f[i] - m * r[i];
     }
 }
 
 // g_new = S(y + c2 u), threshold c2 mu / 2; y <- g_new + beta (g_new - g);
 // g <- g_new. With y == g (ISTA, beta = 0) the update is in place.
-__global__ void __launch_bounds__(kThreads) k_threshold(float* g, float* y, const float* __restrict__ u,
+__global__ void __launch_bounds__(kThreads) k_threshold(float* g, float* y, const float* u,
                                                        float c2, float thr, float beta, long n) {
+    chain_next<8>();
+    chain_wait<8>();
     for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-        const float v = y[i] + c2 * __ldg(u + i);
+        const float v = y[i] + c2 * u[i];
         const float a = fabsf(v) - thr;
         const float gn = a > 0.f ? copysignf(a, v) : 0.f;
         const float go = g[i];
@@ -59,12 +63,14 @@ __global__ void __launch_bounds__(kThreads) k_threshold(float* g, float* y, cons
 
 // Partial sums of squares (FP64) over a grid-stride partition: block b
 // writes part[b]. Fixed grid, fixed order: the sum is deterministic.
-__global__ void __launch_bounds__(kThreads) k_sumsq_partial(const float* __restrict__ x, long n,
-                                                           double* __restrict__ part) {
+__global__ void __launch_bounds__(kThreads) k_sumsq_partial(const float* x, long n,
+                                                           double* part) {
+    chain_next<8>();
+    chain_wait<8>();
     __shared__ double red[kThreads / 32];
     double s = 0.0;
     for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-        const double v = __ldg(x + i);
+        const double v = x[i];
         s += v * v;
     }
 #pragma unroll
@@ -79,7 +85,7 @@ __global__ void __launch_bounds__(kThreads) k_sumsq_partial(const float* __restr
 }
 
 // Sum of the partials, in the same order in every block.
-__device__ __forceinline__ double sum_partials(const double* __restrict__ part, int np) {
+__device__ __forceinline__ double sum_partials(const double* part, int np) {
     __shared__ double tot;
     if (threadIdx.x == 0) {
         double t = 0.0;
@@ -91,9 +97,11 @@ __device__ __forceinline__ double sum_partials(const double* __restrict__ part, 
 }
 
 // y = x / ||x|| (||x|| from the partials); norm_out (if set) = ||x||.
-__global__ void __launch_bounds__(kThreads) k_normalize(const float* __restrict__ x, float* __restrict__ y, long n,
-                                                       const double* __restrict__ part, int np,
-                                                       float* __restrict__ norm_out) {
+__global__ void __launch_bounds__(kThreads) k_normalize(const float* x, float* y, long n,
+                                                       const double* part, int np,
+                                                       float* norm_out) {
+    chain_next<8>();
+    chain_wait<8>();
     const double nrm = sqrt(sum_partials(part, np));
     const float inv = nrm > 0.0 ? (float)(1.0 / nrm) : 0.f;
     if (norm_out && blockIdx.x == 0 && threadIdx.x == 0) *norm_out = (float)nrm;
@@ -107,6 +115,8 @@ __global__ void __launch_bounds__(kThreads) k_normalize(const float* __restrict_
 __global__ void __launch_bounds__(kThreads) k_mute(const float* src, float* dst, int Ntau, long n, double tau0,
                                                   double dtau, double qmin, double dq, const double* qv,
                                                   double q0, double slope, int side) {
+    chain_next<8>();
+    chain_wait<8>();
     for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
         const long l = i / Ntau;
         const double tau = tau0 + dtau * (double)(i - l * Ntau);
@@ -117,10 +127,12 @@ __global__ void __launch_bounds__(kThreads) k_mute(const float* src, float* dst,
 }
 
 // out = a - b, elementwise.
-__global__ void __launch_bounds__(kThreads) k_subtract(const float* __restrict__ a, const float* __restrict__ b,
-                                                      float* __restrict__ out, long n) {
+__global__ void __launch_bounds__(kThreads) k_subtract(const float* a, const float* b,
+                                                      float* out, long n) {
+    chain_next<8>();
+    chain_wait<8>();
     for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
-        out[i] = __ldg(a + i) - __ldg(b + i);
+        out[i] = a[i] - b[i];
 }
 
 int grid_for(long n) {
@@ -179,8 +191,8 @@ extern "C" radon_status radon_ista(radon_plan p, const float* f, const float* ma
     double t = 1.0;
     for (int it = 0; it < iters; ++it) {
         if (radon_status st = radon_adj(p, y, r, stream)) return st;
-        k_residual<<<grid_for(nd), kThreads, 0, s>>>(f, mask, r, d.Nt, nd);
-        if (int e = last_cuda()) return cuda_fail(e, "residual");
+        if (int e = launch_chain(8, k_residual, grid_for(nd), kThreads, 0, stream, f, mask, r, d.Nt, nd))
+            return cuda_fail(e, "residual");
         if (radon_status st = radon_fwd(p, r, u, stream)) return st;
         double beta = 0.0;
         if (accelerate) {
@@ -188,8 +200,8 @@ extern "C" radon_status radon_ista(radon_plan p, const float* f, const float* ma
             beta = (t - 1.0) / tn;
             t = tn;
         }
-        k_threshold<<<grid_for(ni), kThreads, 0, s>>>(g, y, u, c2, thr, (float)beta, ni);
-        if (int e = last_cuda()) return cuda_fail(e, "threshold");
+        if (int e = launch_chain(8, k_threshold, grid_for(ni), kThreads, 0, stream, g, y, u, c2, thr, (float)beta, ni))
+            return cuda_fail(e, "threshold");
     }
     return RADON_OK;
 }
@@ -220,17 +232,18 @@ extern "C" radon_status radon_opnorm(radon_plan p, const float* v0, int iters, f
     float* v = (float*)(w + align256(nd * sizeof(float)));                 // unit vector, [Nq][Ntau]
     float* z = (float*)((char*)v + align256(ni * sizeof(float)));          // R_h R_h* v
     double* part = (double*)((char*)z + align256(ni * sizeof(float)));
-    cudaStream_t s = (cudaStream_t)stream;
-    k_sumsq_partial<<<kNormBlocks, kThreads, 0, s>>>(v0, ni, part);
-    k_normalize<<<grid_for(ni), kThreads, 0, s>>>(v0, v, ni, part, kNormBlocks, nullptr);
-    if (int e = last_cuda()) return cuda_fail(e, "power iteration start");
+    if (int e = launch_chain(8, k_sumsq_partial, kNormBlocks, kThreads, 0, stream, v0, ni, part))
+        return cuda_fail(e, "power iteration start");
+    if (int e = launch_chain(8, k_normalize, grid_for(ni), kThreads, 0, stream, v0, v, ni, part, kNormBlocks, nullptr))
+        return cuda_fail(e, "power iteration start");
     for (int it = 0; it < iters; ++it) {
         if (radon_status st = radon_adj(p, v, a, stream)) return st;
         if (radon_status st = radon_fwd(p, a, z, stream)) return st;
         // ||R R* v|| with ||v|| = 1 tends to the largest eigenvalue of R R*, ||R_h||^2
-        k_sumsq_partial<<<kNormBlocks, kThreads, 0, s>>>(z, ni, part);
-        k_normalize<<<grid_for(ni), kThreads, 0, s>>>(z, v, ni, part, kNormBlocks, norm2);
-        if (int e = last_cuda()) return cuda_fail(e, "power iteration");
+        if (int e = launch_chain(8, k_sumsq_partial, kNormBlocks, kThreads, 0, stream, z, ni, part))
+            return cuda_fail(e, "power iteration");
+        if (int e = launch_chain(8, k_normalize, grid_for(ni), kThreads, 0, stream, z, v, ni, part, kNormBlocks, norm2))
+            return cuda_fail(e, "power iteration");
     }
     return RADON_OK;
 }
@@ -246,9 +259,8 @@ extern "C" radon_status radon_mute(radon_plan p, const float* g, float* out, dou
     radon_desc d;
     radon_plan_desc(p, &d);
     const long ni = (long)d.Nq * d.Ntau;
-    k_mute<<<grid_for(ni), kThreads, 0, (cudaStream_t)stream>>>(g, out, d.Ntau, ni, d.tau0, d.dtau, d.qmin, q_step(d),
-                                                                 plan_q_values(p), q0, slope, side);
-    if (int e = last_cuda()) return cuda_fail(e, "mute");
+    if (int e = launch_chain(8, k_mute, grid_for(ni), kThreads, 0, stream, g, out, d.Ntau, ni, d.tau0, d.dtau, d.qmin, q_step(d), plan_q_values(p), q0, slope, side))
+        return cuda_fail(e, "mute");
     return RADON_OK;
 }
 
@@ -278,7 +290,7 @@ extern "C" radon_status radon_demultiple(radon_plan p, const float* f, double q0
     if (radon_status st = radon_ista(p, f, nullptr, g, iters, c2, mu, accelerate, work, ista_b, stream)) return st;
     if (radon_status st = radon_mute(p, g, gm, q0, slope, RADON_KEEP_ABOVE, stream)) return st;
     if (radon_status st = radon_adj(p, gm, fm, stream)) return st;
-    k_subtract<<<grid_for(nd), kThreads, 0, (cudaStream_t)stream>>>(f, fm, f_out, nd);
-    if (int e = last_cuda()) return cuda_fail(e, "subtraction of the multiples");
+    if (int e = launch_chain(8, k_subtract, grid_for(nd), kThreads, 0, stream, f, fm, f_out, nd))
+        return cuda_fail(e, "subtraction of the multiples");
     return RADON_OK;
 }
