@@ -26,8 +26,15 @@ __all__ = ["Plan", "Batch", "radon", "radon_adjoint", "radon_adj", "direct_forwa
            "HRadon", "default_method"]
 
 
-def _stream_ptr(device: torch.device):
-    return ctypes.c_void_p(torch.cuda.current_stream(device).cuda_stream)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
+def _stream_ptr(device: torch.device) -> int:
+    """The current stream of the device as a pointer. The raw query leaves out
+    the Stream object (2 us of a call's host time)."""
+    if _raw_stream is not None and device.index is not None:
+        return _raw_stream(device.index)
+    return torch.cuda.current_stream(device).cuda_stream
 
 
 def _check_tensor(t: torch.Tensor, shape, name: str, device: torch.device):
@@ -35,7 +42,7 @@ def _check_tensor(t: torch.Tensor, shape, name: str, device: torch.device):
         raise TypeError(f"{name} must be a torch.Tensor")
     if t.device != device or t.dtype != torch.float32 or not t.is_contiguous():
         raise ValueError(f"{name} must be a contiguous float32 tensor on {device}")
-    if tuple(t.shape) != tuple(shape):
+    if t.shape != shape:
         raise ValueError(f"{name} has shape {tuple(t.shape)}, expected {tuple(shape)}")
 
 
@@ -103,6 +110,7 @@ class Plan:
         out = RadonDesc()
         _lib.check(lib.radon_plan_desc(self._handle, ctypes.byref(out)))
         self.desc = out
+        self._fwd, self._adj = lib.radon_fwd, lib.radon_adj
         self.Nt, self.Nx, self.Ntau, self.Nq = Nt, Nx, Ntau, Nq
 
     # -- lifetime ---------------------------------------------------------
@@ -182,9 +190,11 @@ class Plan:
         _check_tensor(f, (self.Nx, self.Nt), "f", self.device)
         if out is None:
             out = torch.empty((self.Nq, self.Ntau), dtype=torch.float32, device=self.device)
-        _check_tensor(out, (self.Nq, self.Ntau), "out", self.device)
-        _lib.check(_lib.load().radon_fwd(self._handle, ctypes.c_void_p(f.data_ptr()),
-                                         ctypes.c_void_p(out.data_ptr()), _stream_ptr(self.device)))
+        else:
+            _check_tensor(out, (self.Nq, self.Ntau), "out", self.device)
+        status = self._fwd(self._handle, f.data_ptr(), out.data_ptr(), _stream_ptr(self.device))
+        if status:
+            _lib.check(status)
         return out
 
     def adjoint(self, g: torch.Tensor, out: torch.Tensor | None = None) -> torch.Tensor:
@@ -192,9 +202,11 @@ class Plan:
         _check_tensor(g, (self.Nq, self.Ntau), "g", self.device)
         if out is None:
             out = torch.empty((self.Nx, self.Nt), dtype=torch.float32, device=self.device)
-        _check_tensor(out, (self.Nx, self.Nt), "out", self.device)
-        _lib.check(_lib.load().radon_adj(self._handle, ctypes.c_void_p(g.data_ptr()),
-                                         ctypes.c_void_p(out.data_ptr()), _stream_ptr(self.device)))
+        else:
+            _check_tensor(out, (self.Nx, self.Nt), "out", self.device)
+        status = self._adj(self._handle, g.data_ptr(), out.data_ptr(), _stream_ptr(self.device))
+        if status:
+            _lib.check(status)
         return out
 
 
