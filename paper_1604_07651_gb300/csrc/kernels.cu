@@ -30,6 +30,7 @@
 #include <type_traits>
 
 #include "device.cuh"
+#include "fft2.cuh"
 
 namespace hr {
 
@@ -198,29 +199,50 @@ __device__ __forceinline__ void grid_merge_split(const PieceDev& P, int4 us, int
     }
     __syncthreads();
     if (!s_last) return;
-    // each thread sums its kCells / kUnitChunks cells over the slots in slot
-    // order, all its cells' loads of two slots in flight together
-    constexpr int kPer = kCells / kUnitChunks;
-    static_assert(kCells % kUnitChunks == 0, "cells per thread");
-    float acc[kPer];
+    // each thread sums two groups of four cells over the slots in slot order,
+    // eight slots' loads in flight (the densest tile of the 2048^2 gather has
+    // 40 slots, and its merge ends the launch)
+    static_assert(kCells == 8 * kUnitChunks, "cells per thread");
+    float4 acc[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+    const float4* src = reinterpret_cast<const float4*>(slot0) + threadIdx.x;
+    for (int u0 = 0; u0 < us.y; u0 += 8) {
+        float4 v[8][2];
 #pragma unroll
-    for (int j = 0; j < kPer; ++j) acc[j] = 0.f;
-    const float* src = slot0 + threadIdx.x;
-#pragma unroll 2
-    for (int u = 0; u < us.y; ++u) {
-        float v[kPer];
+        for (int u = 0; u < 8; ++u)
 #pragma unroll
-        for (int j = 0; j < kPer; ++j) v[j] = __ldcg(src + (size_t)u * kCells + j * kUnitChunks);
+            for (int j = 0; j < 2; ++j)
+                v[u][j] = u0 + u < us.y ? __ldcg(src + (size_t)(u0 + u) * (kCells / 4) + j * kUnitChunks)
+                                        : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int j = 0; j < kPer; ++j) acc[j] += v[j];
+        for (int u = 0; u < 8; ++u)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                acc[j].x += v[u][j].x;
+                acc[j].y += v[u][j].y;
+                acc[j].z += v[u][j].z;
+                acc[j].w += v[u][j].w;
+            }
     }
 #pragma unroll
-    for (int j = 0; j < kPer; ++j) {
-        const int i = threadIdx.x + j * kUnitChunks;
+    for (int j = 0; j < 2; ++j) {
+        const int i = 4 * (threadIdx.x + j * kUnitChunks);
         const int m = i / kTileCols, n = i - m * kTileCols;
-        if (m < nr && n < nc) P.lat[(size_t)(m_lo + m) * P.lp + n_lo + n] = acc[j];
+        // within the row pitch, a multiple of four like n_lo
+        if (m < nr && n < nc) *reinterpret_cast<float4*>(P.lat + (size_t)(m_lo + m) * P.lp + n_lo + n) = acc[j];
     }
     if (threadIdx.x == 0) *counter = 0;
+}
+
+// Cubic tap weights of both axes at once, packed (w1 and w2 as 2/3 - x^2 +
+// x^3 / 2 of x = f and 1 - f): half the instructions of two evaluations.
+__constant__ float2 kSplinePairs[5] = {{0.5f, 0.5f}, {-1.f, -1.f}, {1.0f / 6.0f, 1.0f / 6.0f}, {1.f, 1.f}, {2.f / 3.f, 2.f / 3.f}};
+__device__ __forceinline__ void both_weights(float ft, float fr, float (&wt)[4], float (&wr)[4]) {
+    const f2* k = reinterpret_cast<const f2*>(kSplinePairs);
+    const f2 f = pk(ft, fr), g = sub2(k[3], f), ff = mul2(f, f), gg = mul2(g, g);
+    const float2 w0 = upk(mul2(gg, mul2(g, k[2]))), w3 = upk(mul2(ff, mul2(f, k[2])));
+    const float2 w1 = upk(fma2(ff, fma2(f, k[0], k[1]), k[4])), w2 = upk(fma2(gg, fma2(g, k[0], k[1]), k[4]));
+    wt[0] = w0.x, wt[1] = w1.x, wt[2] = w2.x, wt[3] = w3.x;
+    wr[0] = w0.y, wr[1] = w1.y, wr[2] = w2.y, wr[3] = w3.y;
 }
 
 template <class Src, class T, int NT>
@@ -321,8 +343,12 @@ __global__ void __launch_bounds__(kUnitChunks, NT == 4 ? 4 : 2) k_grid_tiles(con
         wn = n0;
         win = tile + (m0 - m_lo + Tile::halo) * Tile::pitch + n0 - n_lo + Tile::halo;
         float wt[NT], wr[NT];
-        bspline_weights<NT>(__int_as_float(e.y), wt);
-        bspline_weights<NT>(__int_as_float(e.z), wr);
+        if constexpr (NT == 4) {
+            both_weights(__int_as_float(e.y), __int_as_float(e.z), wt, wr);
+        } else {
+            bspline_weights<NT>(__int_as_float(e.y), wt);
+            bspline_weights<NT>(__int_as_float(e.z), wr);
+        }
 #pragma unroll
         for (int a = 0; a < NT; ++a) {
             const float va = v[s] * wt[a];
@@ -867,10 +893,15 @@ int max_smem_optin() {
         }                                                             \
     } while (0)
 
+template <class Src, class T>
+static int launch_grid_as(void (*kern)(Src, const T*), int nb, void* stream, const Src& B, const T* f) {
+    return launch_chain(8, kern, nb, kUnitChunks, 0, stream, B, f);
+}
+
 int launch_grid_tiles(const PieceDev* P, int n, const float* f, void* stream) {
     PieceBatch B;
     const int nb = make_batch(P, n, B, [](const PieceDev& q) { return q.nunits; });
-    if (nb > 0) HR_TAPS(P[0].ntaps, return launch_chain(8, k_grid_tiles<PieceBatch, float, NT>, nb, kUnitChunks, 0, stream, B, f));
+    if (nb > 0) HR_TAPS(P[0].ntaps, return launch_grid_as(k_grid_tiles<PieceBatch, float, NT>, nb, stream, B, f));
     return 0;
 }
 
@@ -878,9 +909,8 @@ int launch_grid_tiles_dev(const DevBatch& S, int nblocks, int ntaps, const void*
     if (nblocks <= 0) return 0;
     HR_TAPS(ntaps, {
         if (in_type == kInBF16)
-            return launch_chain(8, k_grid_tiles<DevBatch, __nv_bfloat16, NT>, nblocks, kUnitChunks, 0, stream, S,
-                                (const __nv_bfloat16*)f);
-        return launch_chain(8, k_grid_tiles<DevBatch, float, NT>, nblocks, kUnitChunks, 0, stream, S, (const float*)f);
+            return launch_grid_as(k_grid_tiles<DevBatch, __nv_bfloat16, NT>, nblocks, stream, S, (const __nv_bfloat16*)f);
+        return launch_grid_as(k_grid_tiles<DevBatch, float, NT>, nblocks, stream, S, (const float*)f);
     });
     return 0;
 }
