@@ -355,7 +355,16 @@ void set_col_groups(PieceDev* P, int n) {
 
 int col_threads(const PieceDev* P, int n) {
     int t = kColThreads;
-    for (int k = 0; k < n; ++k) t = std::max(t, std::min(kColThreadsMax, (P[k].Ptheta / 16 * P[k].C + 31) & ~31));
+    long blocks = 0, most = 0;
+    for (int k = 0; k < n; ++k) {
+        blocks += P[k].nkg;
+        most = std::max<long>(most, P[k].Ptheta / 16 * P[k].C);
+        t = std::max(t, std::min(kColThreadsMax, (P[k].Ptheta / 16 * P[k].C + 31) & ~31));
+    }
+    // short columns that do not fit the chip at once: fewer threads, if that
+    // fits them (the launch's time is then one CTA's latency, not two)
+    for (int s = kColThreads; s >= 64 && t == kColThreads; s -= 32)
+        if (s >= most && blocks > kSMs * (512 / kColThreads) && blocks <= (long)kSMs * (512 / s)) t = s;
     return t;
 }
 
