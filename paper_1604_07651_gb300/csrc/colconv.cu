@@ -37,16 +37,6 @@ constexpr int kColThreadsMax = 384;
 // 480 threads at 128 registers fill the register file: three CTAs of 160, two
 // of 192 to 224, one of 256 and more.
 constexpr int kColThreadsReg = 480;
-// 16-byte asynchronous copies global -> shared (cp.async; the completion
-// wait is the hardware's, no spin loop).
-__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gmem_src) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() {
-    asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
-}
-
 // Twiddles of the middle passes (all but the first and the last), kept in
 // shared memory.
 __host__ __device__ __forceinline__ int col_twiddles(const FftPlan& fp) {

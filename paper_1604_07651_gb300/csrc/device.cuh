@@ -54,6 +54,20 @@ __device__ __forceinline__ unsigned dyn_smem_bytes() {
     return r;
 }
 
+// 16-byte asynchronous copies global -> shared (cp.async; the completion
+// wait is the hardware's, no spin loop).
+__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gmem_src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() {
+    asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+}
+__device__ __forceinline__ void cp_async16_or_zero(void* smem_dst, const void* gmem_src, bool on) {   // zeros unless on
+    const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(gmem_src), "r"(on ? 16 : 0) : "memory");
+}
+
 // Programmatic dependent launch: a kernel of a transform may start while its
 // predecessor on the stream still runs. Each calls chain_wait() before it
 // touches anything another kernel writes (it returns once the predecessor has
