@@ -331,6 +331,7 @@ struct radon_plan_s {
     Grid grid;                                   // given offsets / slownesses (empty: regular)
     const double* q_dev = nullptr;               // [Nq] given slownesses on the device (mute)
     int device = 0;
+    int chunk = 8;                               // most samples of a gridding chunk
     std::vector<HostPiece> pieces;               // slowness-piece major
     std::vector<std::pair<int, int>> qpieces;    // columns of each slowness piece
     std::vector<int> qfirst, qcount;             // pieces of each slowness piece
@@ -655,7 +656,7 @@ radon_status kernel_spectrum(radon_plan_s* p, const HostPiece& h, int nkb, std::
 
 // Tile lists of the forward gridding, built from the device's own position
 // table (copied back once) so that membership matches the kernel exactly:
-// for every tile, the chunks of at most 8 consecutive samples of one trace
+// for every tile, the chunks of at most p->chunk consecutive samples of one trace
 // whose NT x NT footprint meets it (along a trace the footprint moves
 // monotonically, so each trace meets a tile in one run of samples).
 radon_status build_tile_lists(radon_plan_s* p, HostPiece& h, PieceDev& P) {
@@ -678,7 +679,7 @@ radon_status build_tile_lists(radon_plan_s* p, HostPiece& h, PieceDev& P) {
             for (int ti = m0 / TR; ti <= (m0 + NT - 1) / TR && ti < P.ntr; ++ti)
                 for (int tj = n0 / TC; tj <= (n0 + NT - 1) / TC && tj < P.ntc; ++tj) {
                     const int t = ti * P.ntc + tj;
-                    if (last_k[t] == k && last_j[t] == j - 1 && runs[t].back().z < 8) {
+                    if (last_k[t] == k && last_j[t] == j - 1 && runs[t].back().z < p->chunk) {
                         runs[t].back().z += 1;
                     } else {
                         runs[t].push_back(int4{k, j, 1, 0});
@@ -1101,7 +1102,21 @@ static radon_status check_grid(const radon_desc& d, const double* x, const doubl
     return RADON_OK;
 }
 
-static radon_status plan_core(const radon_desc* din, const double* x, const double* q, radon_plan_s** out) {
+// Samples per gridding chunk for launches over `samples` gather samples (one
+// thread grids a chunk, one sample after the other). Four where that still
+// fits the chip at once (four CTAs per SM, two of the quintic kernel; pieces
+// and tiles overlap, so a sample is in about 1.56 chunks): such a launch takes the time of one thread's
+// chain (us per pass, 8 -> 4 samples: 256 x 64 forward 33.3 -> 30.5, FISTA 1024
+// x 256 85.7 -> 80.7 an iteration, 1501 x 233 pair 87.2 -> 85.6). Eight
+// otherwise, with half the window flushes (2048^2 forward 217 against 232).
+static int grid_chunk(double samples, int order) {
+    return 1.56 * samples / 4 <= 152.0 * (order == 5 ? 2 : 4) * kUnitChunks ? 4 : 8;
+}
+
+// launch_samples: gather samples of the launches the plan will be part of (0:
+// its own gather).
+static radon_status plan_core(const radon_desc* din, const double* x, const double* q, double launch_samples,
+                              radon_plan_s** out) {
     *out = nullptr;
     if (radon_status s = check_desc(din)) return s;
     Grid grid;
@@ -1111,6 +1126,7 @@ static radon_status plan_core(const radon_desc* din, const double* x, const doub
     p->d = *din;
     p->grid = std::move(grid);
     radon_desc& d = p->d;
+    p->chunk = grid_chunk(launch_samples > 0 ? launch_samples : (double)d.Nt * d.Nx, d.spline_order);
     if (!p->grid.q.empty()) {            // the descriptor reports the given range
         d.qmin = p->grid.q.front();
         d.qmax = p->grid.q.back();
@@ -1211,7 +1227,7 @@ extern "C" radon_status radon_plan_create_grid(radon_plan* out, const radon_desc
     *out = nullptr;
     arm_alloc_hook();
     radon_plan_s* p = nullptr;
-    if (radon_status s = plan_core(din, x, q, &p)) return s;
+    if (radon_status s = plan_core(din, x, q, 0, &p)) return s;
     DeviceGuard guard(p->device);
     // per-piece work buffers: lattices back to back (one clear per forward),
     // spectra (the column pass works in place), adjoint column profiles
@@ -1687,6 +1703,8 @@ extern "C" radon_status radon_batch_create_grid(radon_batch* out, int n, const r
     // the plans are independent: build them on several host threads (their
     // host-side table work dominates), keeping the first failure
     b->plans.assign(n, nullptr);
+    double samples = 0;
+    for (int i = 0; i < n; ++i) samples += (double)descs[i].Nt * descs[i].Nx;
     std::atomic<int> next{0};
     std::mutex err_mutex;
     radon_status first_err = RADON_OK;
@@ -1696,7 +1714,7 @@ extern "C" radon_status radon_batch_create_grid(radon_batch* out, int n, const r
             radon_desc d = descs[i];
             d.device = b->device;
             radon_plan_s* p = nullptr;
-            if (radon_status s = plan_core(&d, x ? x[i] : nullptr, q ? q[i] : nullptr, &p)) {
+            if (radon_status s = plan_core(&d, x ? x[i] : nullptr, q ? q[i] : nullptr, samples, &p)) {
                 std::lock_guard<std::mutex> lock(err_mutex);
                 if (first_err == RADON_OK) {
                     first_err = s;

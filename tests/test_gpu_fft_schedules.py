@@ -119,3 +119,25 @@ def test_buffers_off_16_bytes(hr, ntau, offset):
     assert torch.equal(plan.adjoint(g, out=view(torch.empty_like(buf), 48, 257)), plan.adjoint(g.clone()))
     assert torch.equal(plan.forward(f, out=view(torch.empty_like(buf), 33, ntau)), plan.forward(f.clone()))
     plan.close()
+
+
+@pytest.mark.parametrize("order", [3, 5])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("gathers", [[(301, 64), (97, 33)], [(1501, 201), (902, 150)]])
+def test_batch_gridding_equals_single_plans(hr, gathers, dtype, order):
+    """A batch's gridding copies its position entries through shared memory
+    and takes chunks of four samples below about 400 000 samples, eight above;
+    single plans of these gathers take four and read their own entries. Both
+    round every contribution to 2^-29 or less of the cell bound (1e-6, as the
+    batches' own tests)."""
+    desc = [dict(Nt=nt, Nx=nx, Ntau=nt - 3, Nq=nx, dt=0.004, dx=0.025, qmin=0.2, qmax=0.7, spline_order=order,
+                 rows_per_band=4) for nt, nx in gathers]
+    gen = torch.Generator(device="cuda").manual_seed(9)
+    fs = [torch.randn((nx, nt), device="cuda", generator=gen).to(dtype) for nt, nx in gathers]
+    batch = hr.Batch(desc)
+    out = batch.unpack_images(batch.forward(batch.pack(fs, dtype=dtype)))
+    for d, f, g in zip(desc, fs, out):
+        plan = hr.Plan(**d)
+        want = plan.forward(f.float())
+        assert float((g - want).norm()) <= 1e-6 * float(want.norm())
+        plan.close()
