@@ -459,11 +459,11 @@ def step_stats(step_ms, event_ms) -> dict:
 
 
 def kernel_source_digest() -> str:
-    """sha256 prefix of the sources the kernels compile from (kernels.cu and
-    the two headers it includes), the key of MEASURED_TRAFFIC."""
+    """sha256 prefix of the sources the kernels compile from, the key of
+    MEASURED_TRAFFIC."""
     import hashlib
     h = hashlib.sha256()
-    for name in ("kernels.cu", "internal.h", "hostdev.h"):
+    for name in ("kernels.cu", "colconv.cu", "rows.cu", "device.cuh", "fft2.cuh", "internal.h", "hostdev.h"):
         with open(os.path.join(ROOT, "paper_1604_07651_gb300", "csrc", name), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
