@@ -143,14 +143,14 @@ PROFILE_EVERY = 4   # eager steps with per-stage kernel events: one per PROFILE_
 
 MEASURED_TRAFFIC = {
     # kernel: (kernel_source_digest() when measured, bytes per launch averaged over a step's launches)
-    "k_grid_tiles": ("0c07c8cc1993e35e", 123.61e6),
-    "k_rows_r2c": ("0c07c8cc1993e35e", 22.00e6),
-    "k_colconv": ("0c07c8cc1993e35e", 47.70e6),
-    "k_rows_c2r": ("0c07c8cc1993e35e", 25.81e6),
-    "k_interp_columns": ("0c07c8cc1993e35e", 94.79e6),
-    "k_col_profiles_cols": ("0c07c8cc1993e35e", 93.55e6),
-    "k_band_rows": ("0c07c8cc1993e35e", 40.35e6),
-    "k_gather_samples": ("0c07c8cc1993e35e", 104.29e6),
+    "k_grid_tiles": ("45a7a83e68fe2ea7", 135.14e6),
+    "k_rows_r2c": ("45a7a83e68fe2ea7", 22.04e6),
+    "k_colconv": ("45a7a83e68fe2ea7", 47.84e6),
+    "k_rows_c2r": ("45a7a83e68fe2ea7", 25.89e6),
+    "k_interp_columns": ("45a7a83e68fe2ea7", 94.61e6),
+    "k_col_profiles_cols": ("45a7a83e68fe2ea7", 92.38e6),
+    "k_band_rows": ("45a7a83e68fe2ea7", 40.24e6),
+    "k_gather_samples": ("45a7a83e68fe2ea7", 102.57e6),
 }
 
 # FFT kernels run out of shared memory and are limited by instruction issue,
