@@ -1105,10 +1105,13 @@ static radon_status check_grid(const radon_desc& d, const double* x, const doubl
 // Samples per gridding chunk for launches over `samples` gather samples (one
 // thread grids a chunk, one sample after the other). Four where that still
 // fits the chip at once (four CTAs per SM, two of the quintic kernel; pieces
-// and tiles overlap, so a sample is in about 1.56 chunks): such a launch takes the time of one thread's
-// chain (us per pass, 8 -> 4 samples: 256 x 64 forward 33.3 -> 30.5, FISTA 1024
-// x 256 85.7 -> 80.7 an iteration, 1501 x 233 pair 87.2 -> 85.6). Eight
-// otherwise, with half the window flushes (2048^2 forward 217 against 232).
+// and tiles overlap, so a sample is in about 1.56 chunks): such a launch takes
+// the time of one thread's chain (us per pass, 8 -> 4 samples: 256 x 64
+// forward 33.3 -> 30.5, FISTA 1024 x 256 85.7 -> 80.7 an iteration, 1501 x 233
+// pair 87.2 -> 85.6, 600 x 600 forward 46.8 -> 42.4, quintic 400 x 300 40.4 ->
+// 37.3). Eight otherwise, with half the window flushes (2048^2 forward 217
+// against 232; 1000 x 800 68.0 against 65.4, quintic 600 x 500 50.4 against
+// 50.7: the line is on the cautious side).
 static int grid_chunk(double samples, int order) {
     return 1.56 * samples / 4 <= 152.0 * (order == 5 ? 2 : 4) * kUnitChunks ? 4 : 8;
 }
