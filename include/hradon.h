@@ -388,7 +388,10 @@ radon_status radon_demultiple(radon_plan p, const float* f, double q0, double sl
  * until the process exits; the plan's own work buffers are not used. Plans
  * whose work memory exceeds it (2048^2 gathers with default parameters need
  * about 76 MB) or that have more than 32 pieces are rejected with
- * RADON_ERR_UNSUPPORTED and a message giving the bytes needed. The first call
+ * RADON_ERR_UNSUPPORTED and a message giving the bytes needed. These count the
+ * buffers without the padding of their rows and with the gridding cut into
+ * runs of 8 samples; where padding or shorter runs take a plan beyond the
+ * array, plan creation has allocated the difference. The first call
  * on a device looks up the array's device address (cudaGetSymbolAddress)
  * with that device current; make that first call before any stream capture.
  * All calls on a device share the one array and it keeps the last call's

@@ -192,9 +192,11 @@ int launch_direct_fwd(const float* f, float* g, int Nt, int Nx, int Ntau, int Nq
 int launch_direct_adj(const float* g, float* f, int Nt, int Nx, int Ntau, int Nq, double dt,
                       double dx, double tau0, double dtau, double qmin, double dq, void* stream);
 
-// Forward transform of a plan with every work buffer carved out of the
+// Forward transform of a plan with its work buffers carved out of the
 // caller-given device area `work` (256-byte aligned, `bytes` long) instead of
-// the plan's own buffers; allocates nothing (plan.cpp). Return radon_status.
+// the plan's own buffers; allocates nothing (plan.cpp). Takes every plan whose
+// plan_forward_work_bytes fit: what row padding and finer work units add to
+// them lies in memory that plan creation set aside. Return radon_status.
 int set_error(int status, const char* msg);   // records the thread's last error, returns status
 int plan_device(const radon_plan_s* p);
 int plan_forward_work_bytes(const radon_plan_s* p, size_t* bytes);

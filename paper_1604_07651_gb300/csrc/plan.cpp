@@ -309,6 +309,7 @@ struct HostPiece {
     std::vector<int> jfirst;
     int max_pairs = 1;                             // most pairs of rows per band shared memory allows
     int max_tile_chunks = 0;                       // most gridding chunks of one tile
+    int slots8 = 0, count8 = 0;                    // partial-tile slots and split tiles with chunks of eight samples
     int order = 3;                                 // B-spline degree
     const int2* lband_R[kMaxBandRows + 1] = {};    // band column ranges for 2, 4, 6 rows per band
     PieceDev dev{};
@@ -347,6 +348,8 @@ struct radon_plan_s {
     int nsblocks = 0;
     int nrho_max = 0;
     size_t interp_limit = 0;                     // shared memory of the output interpolation's profiles
+    char* work_more = nullptr;                   // what radon_fwd_noalloc's static area cannot hold (work_layout)
+    size_t work_more_bytes = 0;
     std::vector<void*> allocs;
     size_t bytes = 0;
     // per-stage timing
@@ -734,6 +737,22 @@ radon_status build_tile_lists(radon_plan_s* p, HostPiece& h, PieceDev& P) {
     // the slots in slot order, so the lattice does not depend on the order in
     // which units run
     for (int t = 0; t < ntiles; ++t) h.max_tile_chunks = std::max(h.max_tile_chunks, (int)runs[t].size());
+    // the same cut into chunks of eight samples, which plan_forward_work_bytes counts
+    for (int t = 0; t < ntiles; ++t) {
+        const std::vector<int4>& r = runs[t];
+        int n8 = 0;
+        for (size_t i = 0; i < r.size();) {
+            int len = r[i].z;
+            size_t j = i + 1;
+            while (j < r.size() && r[j].x == r[i].x && r[j].y == r[i].y + len) len += r[j++].z;
+            n8 += (len + 7) / 8;
+            i = j;
+        }
+        if (n8 > kUnitChunks) {
+            h.slots8 += (n8 + kUnitChunks - 1) / kUnitChunks;
+            h.count8 += 1;
+        }
+    }
     std::vector<int> nper(ntiles, 0), slot0(ntiles, 0), cidx(ntiles, -1), seen(ntiles, 0);
     for (const int4& u : units) nper[u.x]++;
     int nslots = 0, ncount = 0;
@@ -987,6 +1006,51 @@ size_t piece_slot_bytes(const PieceDev& P) { return round256b((size_t)P.nslots *
 size_t piece_spectrum_bytes(const PieceDev& P) { return round256b((size_t)P.nkb * P.sp * sizeof(float4)); }
 size_t piece_profile_bytes(const PieceDev& P) {
     return round256b((size_t)(P.l_hi - P.l_lo + 1) * P.hpitch * sizeof(float));
+}
+
+// Work memory of the forward on caller-given memory, in the order descriptors,
+// lattices (back to back), spectra, slots, each buffer in the caller's area
+// while it has room, else in `more`; descriptors with the pointers go to
+// local (may be null). Returns the bytes of `more` used. What a plan may take
+// (plan_forward_work_bytes) counts neither the rows' padding nor the slots
+// that chunks of four samples add over chunks of eight, so that no choice of
+// layout or work split refuses a plan; for plans near the limit these make
+// up `more`.
+struct WorkHead {
+    PieceDev* pieces;       // device copies of the descriptors
+    float* lat;             // the lattices and counters
+    size_t lat_bytes;
+};
+size_t work_layout(const radon_plan_s* p, char* area, size_t bytes, char* more, PieceDev* local, WorkHead& head) {
+    const int np = (int)p->pieces.size();
+    size_t used = 0, over = 0;
+    auto place = [&](size_t n) -> char* {
+        size_t& at = used + n <= bytes ? used : over;
+        char* base = &at == &used ? area : more;
+        char* r = base ? base + at : nullptr;
+        at += n;
+        return r;
+    };
+    head.lat_bytes = 0;
+    for (auto& h : p->pieces) head.lat_bytes += piece_lattice_bytes(h.dev);
+    head.pieces = (PieceDev*)place(round256b(np * sizeof(PieceDev)));
+    char* lat = place(head.lat_bytes);
+    head.lat = (float*)lat;
+    for (int i = 0; i < np; ++i) {
+        const PieceDev& P = p->pieces[i].dev;
+        char* spec = place(piece_spectrum_bytes(P));
+        if (!local) continue;
+        local[i] = P;
+        local[i].lat = (float*)lat;
+        local[i].spec = (float4*)spec;
+        local[i].prof = nullptr;
+        lat += piece_lattice_bytes(P);
+    }
+    for (int i = 0; i < np; ++i) {
+        char* slots = place(piece_slot_bytes(p->pieces[i].dev));
+        if (local) local[i].slots = (float*)slots;
+    }
+    return over;
 }
 
 // Output columns of a plan for the interpolation kernel: every column of
@@ -1322,6 +1386,19 @@ extern "C" radon_status radon_plan_create_grid(radon_plan* out, const radon_desc
         destroy_plan(p);
         return fail(RADON_ERR_UNSUPPORTED, "too many time pieces for the lattice length along rho "
                                            "(the output interpolation's profiles exceed shared memory)");
+    }
+    // radon_fwd_noalloc takes every plan within its limit
+    size_t need = 0;
+    plan_forward_work_bytes(p, &need);
+    if ((int)p->pieces.size() <= kWorkMaxPieces && need <= RADON_NOALLOC_MAX_BYTES) {
+        WorkHead head;
+        p->work_more_bytes = work_layout(p, nullptr, RADON_NOALLOC_MAX_BYTES, nullptr, nullptr, head);
+        void* more = nullptr;
+        if (p->work_more_bytes && (s = dev_alloc(p, p->work_more_bytes, &more))) {
+            destroy_plan(p);
+            return s;
+        }
+        p->work_more = (char*)more;
     }
     if (cudaDeviceSynchronize() != cudaSuccess) {
         destroy_plan(p);
@@ -1946,11 +2023,9 @@ extern "C" radon_status radon_batch_adj(radon_batch b, const float* g, float* f,
 
 // ---------------------------------------------------------------------------
 // Forward transform on caller-given work memory (used by radon_fwd_noalloc in
-// noalloc.cu). Layout of the area: the device copies of the piece
-// descriptors, every piece's lattice (with its gridding counters) back to
-// back, then every piece's spectrum, then every piece's gridding slots, each
-// 256-byte aligned. Every byte the kernels read there is
-// written earlier in the same call, so nothing has to be cleared beforehand.
+// noalloc.cu), laid out by work_layout in 256-byte units. The lattices and
+// the gridding counters behind them are cleared first; everything else the
+// kernels read there is written earlier in the same call.
 // ---------------------------------------------------------------------------
 namespace hr {
 
@@ -1958,10 +2033,15 @@ int set_error(int status, const char* msg) { return fail((radon_status)status, m
 
 int plan_device(const radon_plan_s* p) { return p->device; }
 
+// 512 bytes of descriptor a piece, lattices and spectra without row padding,
+// slots and counters of chunks of eight samples (work_layout).
 int plan_forward_work_bytes(const radon_plan_s* p, size_t* bytes) {
     if (!p || !bytes) return fail(RADON_ERR_INVALID_ARG, "NULL argument");
-    size_t b = round256b(p->pieces.size() * sizeof(PieceDev));
-    for (auto& h : p->pieces) b += piece_lattice_bytes(h.dev) + piece_spectrum_bytes(h.dev) + piece_slot_bytes(h.dev);
+    size_t b = round256b(p->pieces.size() * 512);
+    for (auto& h : p->pieces)
+        b += round256b((size_t)h.Ntheta * h.Nrho * sizeof(float) + (size_t)h.count8 * sizeof(int)) +
+             round256b((size_t)h.dev.nkb * h.Ntheta * sizeof(float4)) +
+             round256b((size_t)h.slots8 * kTileRows * kTileCols * sizeof(float));
     *bytes = b;
     return RADON_OK;
 }
@@ -1979,33 +2059,16 @@ int plan_forward_in_work(radon_plan_s* p, const float* f, float* g, void* work, 
         return fail(RADON_ERR_UNSUPPORTED,
                     "plan needs " + std::to_string(need) + " bytes of work memory, the area holds " +
                         std::to_string(bytes));
-    char* base = (char*)work;
-    PieceDev* dpieces = (PieceDev*)base;
-    size_t off = round256b(np * sizeof(PieceDev));
-    float* lat = (float*)(base + off);
-    size_t lat_bytes = 0;
     PieceDev local[kWorkMaxPieces];
-    for (int i = 0; i < np; ++i) {
-        local[i] = p->pieces[i].dev;
-        local[i].lat = (float*)(base + off);
-        local[i].prof = nullptr;
-        off += piece_lattice_bytes(local[i]);
-        lat_bytes += piece_lattice_bytes(local[i]);
-    }
-    for (int i = 0; i < np; ++i) {
-        local[i].spec = (float4*)(base + off);
-        off += piece_spectrum_bytes(local[i]);
-    }
-    for (int i = 0; i < np; ++i) {
-        local[i].slots = (float*)(base + off);
-        off += piece_slot_bytes(local[i]);
-    }
+    WorkHead head;
+    if (work_layout(p, (char*)work, bytes, p->work_more, local, head) > p->work_more_bytes)
+        return fail(RADON_ERR_UNSUPPORTED, "the work area is smaller than the one the plan was laid out for");
     DeviceGuard guard(p->device);
-    if (radon_status s = cuda_status(launch_write_pieces(local, np, dpieces, stream), "piece descriptors"))
+    if (radon_status s = cuda_status(launch_write_pieces(local, np, head.pieces, stream), "piece descriptors"))
         return s;
-    if (cudaError_t e = cudaMemsetAsync(lat, 0, lat_bytes, (cudaStream_t)stream))   // the gridding's counters
+    if (cudaError_t e = cudaMemsetAsync(head.lat, 0, head.lat_bytes, (cudaStream_t)stream))   // the gridding's counters
         return cuda_status((int)e, "clearing the work area");
-    return run_forward(p, local, dpieces, f, g, stream);
+    return run_forward(p, local, head.pieces, f, g, stream);
 }
 
 }  // namespace hr
