@@ -43,6 +43,9 @@ struct TableArgs {
     int ntaps;              // B-spline taps per axis: 4 (cubic) or 6 (quintic)
 };
 
+// Row pitch of a lattice, floats: 16-byte rows.
+HD int lat_pitch(int Nrho) { return (Nrho + 3) & ~3; }
+
 // Device-visible description of one sub-problem (one time piece of one
 // slowness piece). Passed to kernels by value.
 struct PieceDev {
@@ -54,7 +57,7 @@ struct PieceDev {
     int C;                  // column blocks per CTA of the column pass
     int nkg;                // its CTAs: ceil(nkb/C)
     int sp;                 // lattice rows between the column blocks of spec (Ntheta, padded)
-    int lp;                 // row pitch of lat, floats: Nrho rounded up to 4
+    int lp;                 // row pitch of lat, floats: lat_pitch(Nrho)
     int Re;                 // lattice rows per band of the row kernels (even: they go in pairs)
     int nbands;
     // samples of the gather

@@ -608,14 +608,16 @@ __global__ void __launch_bounds__(256, NT == 4 ? 8 : 6) k_interp_columns(const P
     const int l = c.z, np = c.y;
     const int Ntau = np_all > 0 ? ntau_all : pieces[c.x].Ntau;
     if (np > kMaxColPieces || (size_t)np * pstride * sizeof(float) > dyn_smem_bytes()) return;
-    // per-piece column data, loaded for all pieces at once
+    // per-piece column data, loaded for all pieces at once (what these arrays
+    // take is not left for the profiles, whose length bounds what a plan may
+    // hold: 448 bytes with four taps, 512 with six)
     __shared__ float4 s_w4[kMaxColPieces];
     __shared__ float2 s_w2[NT > 4 ? kMaxColPieces : 1];
     __shared__ const float* s_r0[kMaxColPieces];
     __shared__ const int2* s_rt[kMaxColPieces];
     __shared__ float s_sc[kMaxColPieces];
     __shared__ int2 s_rg[kMaxColPieces];
-    __shared__ int s_nr[kMaxColPieces], s_lp[kMaxColPieces];
+    __shared__ int s_nr[kMaxColPieces];
     if ((int)threadIdx.x < np) {
         const PieceDev& P = pieces[c.x + threadIdx.x];
         const int lc = l - P.l_lo;
@@ -623,7 +625,6 @@ __global__ void __launch_bounds__(256, NT == 4 ? 8 : 6) k_interp_columns(const P
         if (NT > 4) s_w2[threadIdx.x] = __ldg(P.colw2 + lc);
         s_sc[threadIdx.x] = __ldg(P.colscale + lc);
         s_r0[threadIdx.x] = P.lat + (size_t)__ldg(P.colm0 + lc) * P.lp;
-        s_lp[threadIdx.x] = P.lp;
         s_rt[threadIdx.x] = reinterpret_cast<const int2*>(P.rtab + (size_t)lc * Ntau);
         s_rg[threadIdx.x] = __ldg(P.rrange + lc);
         s_nr[threadIdx.x] = P.Nrho;
@@ -633,12 +634,12 @@ __global__ void __launch_bounds__(256, NT == 4 ? 8 : 6) k_interp_columns(const P
     // profiles, np * pstride floats; four cells per thread and load (the
     // lattice rows are 16-byte aligned), all pieces' loads in flight together
     for (int p = 0; p < np; ++p) {
-        const int Nr = s_nr[p], lp = s_lp[p];
+        const int lp = lat_pitch(s_nr[p]);
         const float4 w4 = s_w4[p];
         const float2 w2 = NT > 4 ? s_w2[p] : make_float2(0.f, 0.f);
         const float* r0 = s_r0[p];
         float* prof = smem_f + p * pstride;
-        for (int n = 4 * threadIdx.x; n < Nr; n += 4 * blockDim.x) {
+        for (int n = 4 * threadIdx.x; n < lp; n += 4 * blockDim.x) {
             float4 a[NT];
 #pragma unroll
             for (int k = 0; k < NT; ++k) a[k] = __ldca(reinterpret_cast<const float4*>(r0 + (size_t)k * lp + n));
@@ -654,6 +655,7 @@ __global__ void __launch_bounds__(256, NT == 4 ? 8 : 6) k_interp_columns(const P
             if (!(pstride & 3)) {
                 *reinterpret_cast<float4*>(prof + n) = v;
             } else {                                   // profiles packed to fit shared memory
+                const int Nr = s_nr[p];
                 prof[n] = v.x;
                 if (n + 1 < Nr) prof[n + 1] = v.y;
                 if (n + 2 < Nr) prof[n + 2] = v.z;

@@ -813,7 +813,7 @@ radon_status build_piece_tables(radon_plan_s* p, HostPiece& h, const std::vector
                         " above the FFT passes' limit (4096, 6144 = 3*2048 or 5120 = 5*1024)");
     P.nkb = (h.k2max + 2) / 2;
     P.sp = (h.Ntheta + 7) & ~7;
-    P.lp = (h.Nrho + 3) & ~3;
+    P.lp = lat_pitch(h.Nrho);
     P.Nt = d.Nt;
     P.Nx = d.Nx;
     P.jt_lo = h.jt_lo;
