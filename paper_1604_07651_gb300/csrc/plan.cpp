@@ -307,6 +307,7 @@ struct HostPiece {
     int n_theta = 0, n_rho = 0, Ntheta = 0, Nrho = 0, Ptheta = 0, Prho = 0, k1max = 0, k2max = 0;
     double dtheta = 0, drho = 0, theta0 = 0, rho0 = 0, theta_m = 0;
     std::vector<int> jfirst;
+    int chunk = 8;                                 // most samples of a gridding chunk
     int max_pairs = 1;                             // most pairs of rows per band shared memory allows
     int max_tile_chunks = 0;                       // most gridding chunks of one tile
     int slots8 = 0, count8 = 0;                    // partial-tile slots and split tiles with chunks of eight samples
@@ -332,7 +333,6 @@ struct radon_plan_s {
     Grid grid;                                   // given offsets / slownesses (empty: regular)
     const double* q_dev = nullptr;               // [Nq] given slownesses on the device (mute)
     int device = 0;
-    int chunk = 8;                               // most samples of a gridding chunk
     std::vector<HostPiece> pieces;               // slowness-piece major
     std::vector<std::pair<int, int>> qpieces;    // columns of each slowness piece
     std::vector<int> qfirst, qcount;             // pieces of each slowness piece
@@ -659,7 +659,7 @@ radon_status kernel_spectrum(radon_plan_s* p, const HostPiece& h, int nkb, std::
 
 // Tile lists of the forward gridding, built from the device's own position
 // table (copied back once) so that membership matches the kernel exactly:
-// for every tile, the chunks of at most p->chunk consecutive samples of one trace
+// for every tile, the chunks of at most h.chunk consecutive samples of one trace
 // whose NT x NT footprint meets it (along a trace the footprint moves
 // monotonically, so each trace meets a tile in one run of samples).
 radon_status build_tile_lists(radon_plan_s* p, HostPiece& h, PieceDev& P) {
@@ -682,7 +682,7 @@ radon_status build_tile_lists(radon_plan_s* p, HostPiece& h, PieceDev& P) {
             for (int ti = m0 / TR; ti <= (m0 + NT - 1) / TR && ti < P.ntr; ++ti)
                 for (int tj = n0 / TC; tj <= (n0 + NT - 1) / TC && tj < P.ntc; ++tj) {
                     const int t = ti * P.ntc + tj;
-                    if (last_k[t] == k && last_j[t] == j - 1 && runs[t].back().z < p->chunk) {
+                    if (last_k[t] == k && last_j[t] == j - 1 && runs[t].back().z < h.chunk) {
                         runs[t].back().z += 1;
                     } else {
                         runs[t].push_back(int4{k, j, 1, 0});
@@ -788,8 +788,7 @@ radon_status build_tile_lists(radon_plan_s* p, HostPiece& h, PieceDev& P) {
     return RADON_OK;
 }
 
-radon_status build_piece_tables(radon_plan_s* p, HostPiece& h, const std::vector<double>& bs,
-                                const std::vector<double>& phi_all, int smem_max) {
+radon_status build_piece_tables(radon_plan_s* p, HostPiece& h, const std::vector<double>& bs, int smem_max) {
     const radon_desc& d = p->d;
     const double n_t = d.Nt - 1, n_x = d.Nx - 1;
     const double T = n_t * d.dt, X = offset_X(d, p->grid);
@@ -1166,24 +1165,37 @@ static radon_status check_grid(const radon_desc& d, const double* x, const doubl
     return RADON_OK;
 }
 
-// Samples per gridding chunk for launches over `samples` gather samples (one
-// thread grids a chunk, one sample after the other). Four where that still
-// fits the chip at once (four CTAs per SM, two of the quintic kernel; pieces
-// and tiles overlap, so a sample is in about 1.56 chunks): such a launch takes
-// the time of one thread's chain (us per pass, 8 -> 4 samples: 256 x 64
-// forward 33.3 -> 30.5, FISTA 1024 x 256 85.7 -> 80.7 an iteration, 1501 x 233
-// pair 87.2 -> 85.6, 600 x 600 forward 46.8 -> 42.4, quintic 400 x 300 40.4 ->
-// 37.3). Eight otherwise, with half the window flushes (2048^2 forward 217
-// against 232; 1000 x 800 68.0 against 65.4, quintic 600 x 500 50.4 against
-// 50.7: the line is on the cautious side).
-static int grid_chunk(double samples, int order) {
-    return 1.56 * samples / 4 <= 152.0 * (order == 5 ? 2 : 4) * kUnitChunks ? 4 : 8;
+// Samples per gridding chunk of the pieces of one launch that grids `samples`
+// samples (piece_samples; one thread grids a chunk, one sample after the
+// other, and a sample is in about 1.18 chunks, the tiles' overlap). Four in
+// launches of up to about 730 work units: they take the time of one thread's
+// chain (us per pass, 8 -> 4 samples: 256 x 64 forward 33.3 -> 30.5, FISTA
+// 1024 x 256 85.7 -> 80.7 an iteration, 1501 x 233 pair 87.2 -> 85.6, 600 x
+// 600 forward 46.9 -> 42.5, 1500 x 300 47.6 -> 46.3, quintic 400 x 300 40.4 ->
+// 37.2, but 600 x 500 50.1 -> 50.8). Eight above, with half the window flushes and half the partial tiles
+// (800 x 700 51.2 against 51.2, 900 x 700 56.0 against 58.2, 2048^2 forward
+// 217 against 232, quintic 600 x 500 in two slowness pieces 63.0 against 66.8).
+// A launch holds kMaxBatch pieces of a plan: with several slowness pieces the
+// full launches may take eight and what is left over four (1024 x 256 in three
+// slowness pieces: eight in both launches 85.2, eight and four 80.1, four in
+// both 80.4; in eight slowness pieces 149, 166, 174; 600 x 600 in four 103,
+// 107, 116). The kernel of a batch (all its pieces in one launch) has five
+// cubic CTAs per SM: eight from the units that fill four, two of the quintic
+// one (gathers of 1501 x 201 and 902 x 150 50.1 against 52.2; 520 x 72 and
+// three smaller ones four: 37.4 against 39.5).
+static int grid_chunk(double samples, int order, bool batch) {
+    const double most = !batch ? 1.2 * 4 : order == 5 ? 2 : 4;       // units per SM
+    return 1.18 * samples / 4 <= 152 * most * kUnitChunks ? 4 : 8;
+}
+static double piece_samples(const HostPiece& h) {      // the samples of its time range that are not muted
+    double n = 0;
+    for (int j : h.jfirst) n += h.jt_hi - j + 1;
+    return n;
 }
 
-// launch_samples: gather samples of the launches the plan will be part of (0:
-// its own gather).
-static radon_status plan_core(const radon_desc* din, const double* x, const double* q, double launch_samples,
-                              radon_plan_s** out) {
+// A plan's descriptor and the geometry of its pieces, before anything on the
+// device.
+static radon_status plan_geometry(const radon_desc* din, const double* x, const double* q, radon_plan_s** out) {
     *out = nullptr;
     if (radon_status s = check_desc(din)) return s;
     Grid grid;
@@ -1193,7 +1205,6 @@ static radon_status plan_core(const radon_desc* din, const double* x, const doub
     p->d = *din;
     p->grid = std::move(grid);
     radon_desc& d = p->d;
-    p->chunk = grid_chunk(launch_samples > 0 ? launch_samples : (double)d.Nt * d.Nx, d.spline_order);
     if (!p->grid.q.empty()) {            // the descriptor reports the given range
         d.qmin = p->grid.q.front();
         d.qmax = p->grid.q.back();
@@ -1214,19 +1225,14 @@ static radon_status plan_core(const radon_desc* din, const double* x, const doub
     } else {
         p->device = d.device;
     }
-    DeviceGuard guard(p->device);
-    const int smem_max = max_smem_optin();
-    const std::vector<double> bs = accepted_splits(d);
-    const std::vector<TPiece> tps = time_pieces(d, bs);
+    const std::vector<TPiece> tps = time_pieces(d, accepted_splits(d));
     p->qpieces = slowness_pieces(d, p->grid);
     std::vector<double> phi_all;
     for (auto& lq : p->qpieces) {
         p->qfirst.push_back((int)p->pieces.size());
         for (auto& tp : tps) {
             HostPiece h;
-            radon_status s = make_geometry(d, p->grid, tp, lq, h, phi_all);
-            if (s == RADON_OK) s = build_piece_tables(p, h, bs, phi_all, smem_max);
-            if (s != RADON_OK) {
+            if (radon_status s = make_geometry(d, p->grid, tp, lq, h, phi_all)) {
                 destroy_plan(p);
                 return s;
             }
@@ -1234,6 +1240,20 @@ static radon_status plan_core(const radon_desc* din, const double* x, const doub
         }
         p->qcount.push_back((int)tps.size());
     }
+    *out = p;
+    return RADON_OK;
+}
+
+// The tables and kernel spectra of every piece; destroys the plan on failure.
+static radon_status plan_tables(radon_plan_s* p) {
+    DeviceGuard guard(p->device);
+    const int smem_max = max_smem_optin();
+    const std::vector<double> bs = accepted_splits(p->d);
+    for (auto& h : p->pieces)
+        if (radon_status s = build_piece_tables(p, h, bs, smem_max)) {
+            destroy_plan(p);
+            return s;
+        }
     for (auto& h : p->pieces) p->nrho_max = std::max(p->nrho_max, h.dev.Nrho);
     if (!p->grid.q.empty()) {
         if (radon_status s = dev_upload(p, p->grid.q, &p->q_dev)) {
@@ -1241,7 +1261,6 @@ static radon_status plan_core(const radon_desc* din, const double* x, const doub
             return s;
         }
     }
-    *out = p;
     return RADON_OK;
 }
 
@@ -1294,7 +1313,14 @@ extern "C" radon_status radon_plan_create_grid(radon_plan* out, const radon_desc
     *out = nullptr;
     arm_alloc_hook();
     radon_plan_s* p = nullptr;
-    if (radon_status s = plan_core(din, x, q, 0, &p)) return s;
+    if (radon_status s = plan_geometry(din, x, q, &p)) return s;
+    for (size_t i = 0; i < p->pieces.size(); i += kMaxBatch) {      // one launch each
+        const size_t e = std::min(p->pieces.size(), i + kMaxBatch);
+        double samples = 0;
+        for (size_t k = i; k < e; ++k) samples += piece_samples(p->pieces[k]);
+        for (size_t k = i; k < e; ++k) p->pieces[k].chunk = grid_chunk(samples, p->d.spline_order, false);
+    }
+    if (radon_status s = plan_tables(p)) return s;
     DeviceGuard guard(p->device);
     // per-piece work buffers: lattices back to back (one clear per forward),
     // spectra (the column pass works in place), adjoint column profiles
@@ -1781,36 +1807,51 @@ extern "C" radon_status radon_batch_create_grid(radon_batch* out, int n, const r
         return fail(RADON_ERR_CUDA, "no CUDA device");
     }
     // the plans are independent: build them on several host threads (their
-    // host-side table work dominates), keeping the first failure
+    // host-side table work dominates), keeping the first failure; the tables
+    // need the samples that the batch's launches hold
     b->plans.assign(n, nullptr);
-    double samples = 0;
-    for (int i = 0; i < n; ++i) samples += (double)descs[i].Nt * descs[i].Nx;
-    std::atomic<int> next{0};
-    std::mutex err_mutex;
     radon_status first_err = RADON_OK;
     std::string first_msg;
-    auto worker = [&]() {
-        for (int i = next++; i < n; i = next++) {
-            radon_desc d = descs[i];
-            d.device = b->device;
-            radon_plan_s* p = nullptr;
-            if (radon_status s = plan_core(&d, x ? x[i] : nullptr, q ? q[i] : nullptr, samples, &p)) {
-                std::lock_guard<std::mutex> lock(err_mutex);
-                if (first_err == RADON_OK) {
-                    first_err = s;
-                    first_msg = "gather " + std::to_string(i) + ": " + g_err;
+    auto on_threads = [&](auto&& build) {          // build(i): the status of gather i
+        std::atomic<int> next{0};
+        std::mutex err_mutex;
+        auto worker = [&]() {
+            for (int i = next++; i < n; i = next++)
+                if (radon_status s = build(i)) {
+                    std::lock_guard<std::mutex> lock(err_mutex);
+                    if (first_err == RADON_OK) {
+                        first_err = s;
+                        first_msg = "gather " + std::to_string(i) + ": " + g_err;
+                    }
+                    next = n;
+                    return;
                 }
-                next = n;
-                return;
-            }
-            b->plans[i] = p;
-        }
+        };
+        const int nthreads =
+            std::max(1, std::min<int>(n, std::min(16u, std::max(1u, std::thread::hardware_concurrency()))));
+        std::vector<std::thread> pool;
+        for (int t = 1; t < nthreads; ++t) pool.emplace_back(worker);
+        worker();
+        for (auto& t : pool) t.join();
+        return first_err;
     };
-    const int nthreads = std::max(1, std::min<int>(n, std::min(16u, std::max(1u, std::thread::hardware_concurrency()))));
-    std::vector<std::thread> pool;
-    for (int t = 1; t < nthreads; ++t) pool.emplace_back(worker);
-    worker();
-    for (auto& t : pool) t.join();
+    on_threads([&](int i) {
+        radon_desc d = descs[i];
+        d.device = b->device;
+        return plan_geometry(&d, x ? x[i] : nullptr, q ? q[i] : nullptr, &b->plans[i]);
+    });
+    if (first_err == RADON_OK) {
+        double samples = 0;
+        for (radon_plan_s* p : b->plans)
+            for (auto& h : p->pieces) samples += piece_samples(h);
+        for (radon_plan_s* p : b->plans)
+            for (auto& h : p->pieces) h.chunk = grid_chunk(samples, p->d.spline_order, true);
+        on_threads([&](int i) {
+            const radon_status s = plan_tables(b->plans[i]);
+            if (s) b->plans[i] = nullptr;
+            return s;
+        });
+    }
     if (first_err != RADON_OK) {
         destroy_batch(b);
         return fail(first_err, first_msg);
