@@ -59,6 +59,16 @@ HD void bspline_weights<4>(float f, float w[4]) { b3_weights(f, w); }
 template <>
 HD void bspline_weights<6>(float f, float w[6]) { b5_weights(f, w); }
 
+// Arrival of one of a tile's `units` at its counter; true for the last. `inc`
+// counts like CUDA's atomicInc: returns the old value and stores it plus one,
+// or zero where it has reached the argument. So the counter holds zero again
+// after every full round without a store of its own, also when the rounds of
+// calls that wrongly overlap on one plan mix (their results are lost, the
+// plan is not: a store of zero by the last unit could fall between the other
+// call's arrivals and leave a count behind for good).
+template <class Inc>
+HD bool last_arrival(int units, Inc&& inc) { return inc((unsigned)units - 1) == (unsigned)units - 1; }
+
 // Shared-memory layout of every FFT buffer: element i of a sequence lives at
 // sw(i). XOR-ing the low four bits with the next four spreads the strided
 // stores of the first radix-16 stage (stride 16 elements) over all banks and

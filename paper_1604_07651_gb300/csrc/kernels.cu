@@ -177,8 +177,9 @@ __device__ __forceinline__ void slide_cols_left(int* t, float (&acc)[NT * NT]) {
 // Split tiles: the unit's partial tile (value(i) of cell i, row-major over
 // the kTileRows x kTileCols cells) goes to its slot; the unit that finds it
 // is the tile's last to arrive (the others' slots are then complete and
-// visible) sums every slot of the tile in slot order into the lattice and
-// clears the counter. The result does not depend on which unit runs first.
+// visible) sums every slot of the tile in slot order into the lattice. The
+// result does not depend on which unit runs first; the counter is back at zero
+// once every unit has arrived (last_arrival).
 // Ordering: the block's slot stores, a barrier, then one thread's fence and
 // count (release, cumulative over the block through the barrier); on the
 // reading side that thread's fence after the count, a barrier, and L2 loads.
@@ -190,10 +191,10 @@ __device__ __forceinline__ void grid_merge_split(const PieceDev& P, int4 us, int
     float* slot0 = P.slots + (size_t)us.x * kCells;
     for (int i = threadIdx.x; i < kCells; i += blockDim.x) slot0[(size_t)us.z * kCells + i] = value(i);
     __syncthreads();
-    int* counter = reinterpret_cast<int*>(P.lat + (size_t)P.Ntheta * P.lp) + us.w;
+    unsigned* counter = reinterpret_cast<unsigned*>(P.lat + (size_t)P.Ntheta * P.lp) + us.w;
     if (threadIdx.x == 0) {
         __threadfence();
-        const int last = atomicAdd(counter, 1) == us.y - 1;
+        const bool last = last_arrival(us.y, [&](unsigned most) { return atomicInc(counter, most); });
         if (last) __threadfence();
         s_last = last;
     }
@@ -230,7 +231,6 @@ __device__ __forceinline__ void grid_merge_split(const PieceDev& P, int4 us, int
         // within the row pitch, a multiple of four like n_lo
         if (m < nr && n < nc) *reinterpret_cast<float4*>(P.lat + (size_t)(m_lo + m) * P.lp + n_lo + n) = acc[j];
     }
-    if (threadIdx.x == 0) *counter = 0;
 }
 
 // Cubic tap weights of both axes at once, packed (w1 and w2 as 2/3 - x^2 +
