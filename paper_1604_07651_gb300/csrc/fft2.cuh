@@ -128,15 +128,13 @@ __device__ __forceinline__ c2 conj_subi(c2 a, c2 b) { return {add2(a.re, b.im), 
 
 // --------------------------------------------------------------------------
 // Passes of the in-place FFT pair (dif_plan) on sequences of 16-byte elements
-// in shared memory. Element i lives at pad(i) = i + i / 16 + i / S0 (S0 the
-// first pass's stride, a multiple of 16): the quarter warps of every pass (consecutive elements, stride 16, and the stride-1
-// pass's 16 elements per thread) touch eight different 16-byte bank groups,
-// and for a stride S < S0 that is a multiple of 16 the addresses of a
-// butterfly advance by the constant S + S / 16, those of the first pass by S0
-// + S0 / 16 + 1 (the odd step spreads the frequencies of neighbouring digits,
-// which the row kernels read and write, over the banks). Sequences of n
-// elements (n a multiple of 16) back to back are one sequence for every pass
-// but the first and last.
+// in shared memory, element i at padn(i) = i + i / 16 + i / S0 (hostdev.h; S0
+// the first pass's stride): the quarter warps of every pass (consecutive
+// elements, stride 16, and the stride-1 pass's 16 elements per thread) touch
+// eight different 16-byte bank groups, and the odd step of the first pass
+// spreads the frequencies of neighbouring digits, which the row kernels read
+// and write, over the banks. Sequences of n elements (n a multiple of 16) back
+// to back are one sequence for every pass but the first and last.
 //
 // Every stride is a power of two (the factor 3, 5 or 9 is in pass 0), and a
 // length that is a multiple of 16 and longer ends with a radix-16 pass of
@@ -154,15 +152,6 @@ __device__ __forceinline__ c2 conj_subi(c2 a, c2 b) { return {add2(a.re, b.im), 
 // the forward butterflies and twiddles on exchanged data; the exchange itself
 // is a renaming where data enter and leave.
 // --------------------------------------------------------------------------
-HD int pad16(int i) { return i + (i >> 4); }                  // pass_any's layout
-HD int padn(int i, int ls0) { return i + (i >> 4) + (i >> ls0); }
-HD int first_step(int ls0) { return (1 << ls0) + (1 << ls0 >> 4) + 1; }
-// Lengths the passes with these address rules serve; the others (small ones)
-// take pass_any.
-HD bool fft_by16(int n) { return n >= 32 && (n & 15) == 0; }
-// Elements between sequences of length n in shared memory.
-HD int seq_pitch(int n, int R0) { return fft_by16(n) ? n + (n >> 4) + R0 : n + (n >> 4) + 1; }
-
 // Twiddle product of a butterfly: x[k] *= T[(k - 1) S] (T at the butterfly's
 // m; entries (wr, wr, wi, wi)).
 template <int R>

@@ -69,18 +69,15 @@ HD void bspline_weights<6>(float f, float w[6]) { b5_weights(f, w); }
 template <class Inc>
 HD bool last_arrival(int units, Inc&& inc) { return inc((unsigned)units - 1) == (unsigned)units - 1; }
 
-// Shared-memory layout of every FFT buffer: element i of a sequence lives at
-// sw(i). XOR-ing the low four bits with the next four spreads the strided
-// stores of the first radix-16 stage (stride 16 elements) over all banks and
-// keeps contiguous accesses conflict-free. A permutation within each block of
-// 16 (and the identity below 16), so sw(i) < n for every length the FFT uses.
+// A layout of 8-byte elements that no kernel uses any more (tests/hostdev_check.cpp
+// still checks it): the low four bits XOR-ed with the next four, a permutation
+// within each block of 16 (and the identity below 16).
 HD int sw(int i) { return i ^ ((i >> 4) & 15); }
 
 HD cf cmul(cf a, cf b) { return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x}; }
 HD cf cmulc(cf a, cf b) { return {a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y}; }  // a * conj(b)
 HD cf cadd(cf a, cf b) { return {a.x + b.x, a.y + b.y}; }
 HD cf csub(cf a, cf b) { return {a.x - b.x, a.y - b.y}; }
-HD cf cconj(cf a) { return {a.x, -a.y}; }
 // The operations of the in-register DFTs, on one complex number (cf) here and
 // on the same element of two sequences at once in the kernels (fft2.cuh):
 // a + i b, a - i b, the product with a constant, a + s b and s a for real s.
@@ -532,11 +529,8 @@ HD int dif_plan(int n, int R[kMaxDifPasses], int S[kMaxDifPasses]) {
     return s;
 }
 
-// Shared-memory layout of the 16-byte elements (two spectrum columns) of the
-// column kernel: the low three bits of the index are XOR-ed with bits 4..6,
-// so that the 8 elements of a quarter warp land in 8 different 16-byte bank
-// groups both for consecutive indices and for the stride-16 accesses of a
-// radix-16 pass. Changes only the low three bits: a permutation of every
+// A layout of 16-byte elements that no kernel uses any more either (padn took
+// its place): the low three bits XOR-ed with bits 4..6, a permutation of every
 // aligned group of 8 (and the identity below 16).
 HD int swc(int i) { return i ^ ((i >> 4) & 7); }
 
@@ -570,6 +564,43 @@ HD int dif_pos(int s, const int R[kMaxDifPasses], const int S[kMaxDifPasses], in
     }
     return pos;
 }
+
+// Shared-memory layouts of the kernels' sequences of 16-byte elements (the same
+// element of two columns or rows, fft2.cuh). Lengths of 32 and more that are
+// multiples of 16: element i at padn(i) = i + i / 16 + i / S0, S0 = 1 << ls0
+// the first pass's stride (a multiple of 16). For a pass of stride S < S0, a
+// multiple of 16, the addresses of a butterfly advance by the constant S + S /
+// 16, those of the first pass by first_step, those of the last pass by one.
+// The other lengths (small ones): pad16.
+HD int pad16(int i) { return i + (i >> 4); }
+HD int padn(int i, int ls0) { return i + (i >> 4) + (i >> ls0); }
+HD int first_step(int ls0) { return (1 << ls0) + (1 << ls0 >> 4) + 1; }
+HD bool fft_by16(int n) { return n >= 32 && (n & 15) == 0; }
+// Elements between sequences of length n, R0 the first pass's radix.
+HD int seq_pitch(int n, int R0) { return fft_by16(n) ? n + (n >> 4) + R0 : n + (n >> 4) + 1; }
+
+// padn(dif_pos(k)) of a length fft_by16 serves: the digits of k times padded
+// strides. lst: log2 of the strides.
+struct FreqDigits {
+    unsigned magic;          // ceil(2^20 / R0): k / R0 = (k magic) >> 20, exact while the product fits 32 bits, k < 2^12 R0
+    int R0, step0, l1, l2, step1, s;
+    HD FreqDigits(int passes, int radix0, const int* lst) {
+        R0 = radix0;
+        magic = ((1u << 20) + R0 - 1) / R0;
+        s = passes;
+        step0 = first_step(lst[0]);
+        l1 = lst[0] - lst[1];                        // log2 of the second radix
+        step1 = (1 << lst[1]) + (1 << lst[1] >> 4);
+        l2 = s > 2 ? lst[1] - lst[2] : 0;            // log2 of the third
+    }
+    HD int operator()(int k) const {
+        const int q = (int)(((unsigned)k * magic) >> 20), k0 = k - q * R0;
+        if (s == 2) return k0 * step0 + q;
+        const int k1 = q & ((1 << l1) - 1), r = q >> l1;
+        if (s == 3) return k0 * step0 + k1 * step1 + r;
+        return k0 * step0 + k1 * step1 + (r & ((1 << l2) - 1)) * 17 + (r >> l2);
+    }
+};
 
 // Every pass's twiddle table back to back in pass order (the last pass has
 // none); returns the number of entries (T may be null to query it).

@@ -907,7 +907,7 @@ radon_status build_piece_tables(radon_plan_s* p, HostPiece& h, const std::vector
     {
         int R[kMaxDifPasses], S[kMaxDifPasses];
         const int s = dif_plan(M, R, S);
-        for (int k = 0; k < M; ++k) rpos[k] = dif_pos(s, R, S, k) + dif_pos(s, R, S, k) / 16;   // pad16
+        for (int k = 0; k < M; ++k) rpos[k] = pad16(dif_pos(s, R, S, k));
     }
     for (int k = 0; k <= M; ++k)
         twP[k] = {(float)std::cos(-2 * kPi * k / h.Prho), (float)std::sin(-2 * kPi * k / h.Prho)};

@@ -146,32 +146,15 @@ __device__ __forceinline__ void row_passes_any(c2* A, int pitch, const FftPlan& 
     }
 }
 
-// Where the forward passes leave frequency k (dif_pos): digits of k times
-// padded strides, for lengths fft_by16 serves computed (a table read would put
-// its latency before every access), else from the plan's table.
+// Where the forward passes leave frequency k (dif_pos): for lengths fft_by16
+// serves computed (a table read would put its latency before every access),
+// else from the plan's table.
 struct FreqPos {
     const int* tab;
-    unsigned magic;          // ceil(2^20 / R0): k / R0 = (k magic) >> 20, exact for k < 2^16
-    int R0, step0, l1, l2, step1, s;
-    __device__ __forceinline__ FreqPos(const PieceDev& P) {
-        const FftPlan& fp = P.fftM;
-        tab = fft_by16(fp.n) ? nullptr : P.rpos;
-        R0 = fp.rad[0];
-        magic = ((1u << 20) + R0 - 1) / R0;
-        s = fp.nst;
-        step0 = first_step(fp.lst[0]);
-        l1 = fp.lst[0] - fp.lst[1];                  // log2 of the second radix
-        step1 = (1 << fp.lst[1]) + (1 << fp.lst[1] >> 4);
-        l2 = s > 2 ? fp.lst[1] - fp.lst[2] : 0;      // log2 of the third
-    }
-    __device__ __forceinline__ int operator()(int k) const {
-        if (tab) return __ldg(tab + k);
-        const int q = (int)(((unsigned)k * magic) >> 20), k0 = k - q * R0;
-        if (s == 2) return k0 * step0 + q;
-        const int k1 = q & ((1 << l1) - 1), r = q >> l1;
-        if (s == 3) return k0 * step0 + k1 * step1 + r;
-        return k0 * step0 + k1 * step1 + (r & ((1 << l2) - 1)) * 17 + (r >> l2);
-    }
+    FreqDigits digits;
+    __device__ __forceinline__ FreqPos(const PieceDev& P)
+        : tab(fft_by16(P.fftM.n) ? nullptr : P.rpos), digits(P.fftM.nst, P.fftM.rad[0], P.fftM.lst) {}
+    __device__ __forceinline__ int operator()(int k) const { return tab ? __ldg(tab + k) : digits(k); }
 };
 
 // Real-FFT post-processing of the band's transformed rows into the half

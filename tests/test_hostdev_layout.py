@@ -25,3 +25,18 @@ def test_arrivals_at_a_split_tile(results):
     """After any number of rounds at a counter, overlapping ones too, the next
     round's last unit is found and no other."""
     assert results["arrival_violations"] == 0
+
+
+def test_shared_memory_layouts(results):
+    """Every FFT length: elements within their pitch and apart, sequences back
+    to back, the constant address steps of each pass, and the computed
+    positions of the frequencies."""
+    # 2^a <= 4096 but 1, which has no pass, 3 2^a <= 6144, 5 2^a <= 5120, 9 2^a <= 2304: 12 + 12 + 11 + 9
+    assert results["fft_lengths"] == 44
+    assert results["layout_violations"] == 0
+
+
+def test_dfts_that_skip_zero_inputs(results):
+    """First-pass butterflies of every radix, with all inputs and with the
+    upper half zero, against the definition: a few roundings of 6e-8 each."""
+    assert results["dft_zeros_rel_l2"] < 5e-7
