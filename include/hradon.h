@@ -76,11 +76,16 @@ typedef struct radon_plan_s* radon_plan;
  *   n_qsplit: number of slowness pieces (Section 5), >= 1; each gets its
  *             own log-polar setup.
  *   device  : CUDA device ordinal, or -1 for the calling thread's current device.
- *   rows_per_band: lattice rows one CTA of the row-FFT kernels holds, 1..6,
- *             or 0 to have radon_plan_create_ex (and radon_batch_create, when
- *             every descriptor asks for it) time each feasible value on the
- *             device and keep the fastest; radon_plan_desc reports the choice.
- *             It changes the work split only, not the results.
+ *   rows_per_band: lattice rows one CTA of the row-FFT kernels is to hold,
+ *             1..6, or 0 to have radon_plan_create_ex (and radon_batch_create,
+ *             when every descriptor asks for it) time 2, 4 and 6, as far as
+ *             feasible, on the device and keep the fastest. Rows go in pairs:
+ *             an odd value runs as the next even one (in a single plan whose
+ *             lattices have too few rows for two CTAs per SM, 3 and 5 as the
+ *             even one below), and a value that shared memory cannot hold as
+ *             the largest that it can. radon_plan_desc reports the value
+ *             asked for, or the one found by timing. It changes the work
+ *             split only, not the results.
  *   spline_order: degree of the B-spline of the gridding, the deconvolution
  *             and the interpolation (Eq. (14)-(17)): 3 (cubic, the default)
  *             or 5 (quintic, the higher-order kernel of Section 7: six taps

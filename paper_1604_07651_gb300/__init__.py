@@ -64,8 +64,10 @@ class Plan:
     (``dtau=0``: ``(Nt-1) dt/(Ntau-1)``) and ``q`` evenly on
     ``[qmin, qmax]``; method parameters ``sigma``, ``omega_c``, ``tsplit``
     (split points of Eq. (19) as fractions of T), ``n_qsplit``;
-    ``rows_per_band`` (1..6, or 0 to time them at plan creation; the plan's
-    ``desc.rows_per_band`` reports the value in use); ``spline_order`` 3
+    ``rows_per_band`` (1..6, or 0 to time 2, 4 and 6 at plan creation; rows go
+    in pairs, so an odd value runs as an even one next to it, and
+    ``desc.rows_per_band`` reports the value asked for or found by timing);
+    ``spline_order`` 3
     (cubic B-splines, the default) or 5 (quintic). Unequally spaced grids
     (``radon_plan_create_grid``): ``x`` gives the Nx offsets (km) in place of
     ``k*dx``, ``q`` the Nq slownesses (s/km) in place of the regular grid.
