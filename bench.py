@@ -143,14 +143,14 @@ PROFILE_EVERY = 4   # eager steps with per-stage kernel events: one per PROFILE_
 
 MEASURED_TRAFFIC = {
     # kernel: (kernel_source_digest() when measured, bytes per launch averaged over a step's launches)
-    "k_grid_tiles": ("45a7a83e68fe2ea7", 135.14e6),
-    "k_rows_r2c": ("45a7a83e68fe2ea7", 22.04e6),
-    "k_colconv": ("45a7a83e68fe2ea7", 47.84e6),
-    "k_rows_c2r": ("45a7a83e68fe2ea7", 25.89e6),
-    "k_interp_columns": ("45a7a83e68fe2ea7", 94.61e6),
-    "k_col_profiles_cols": ("45a7a83e68fe2ea7", 92.38e6),
-    "k_band_rows": ("45a7a83e68fe2ea7", 40.24e6),
-    "k_gather_samples": ("45a7a83e68fe2ea7", 102.57e6),
+    "k_grid_tiles": ("6ea5681c1658f311", 135.36e6),
+    "k_rows_r2c": ("6ea5681c1658f311", 22.04e6),
+    "k_colconv": ("6ea5681c1658f311", 47.84e6),
+    "k_rows_c2r": ("6ea5681c1658f311", 25.89e6),
+    "k_interp_columns": ("6ea5681c1658f311", 94.91e6),
+    "k_col_profiles_cols": ("6ea5681c1658f311", 92.21e6),
+    "k_band_rows": ("6ea5681c1658f311", 40.28e6),
+    "k_gather_samples": ("6ea5681c1658f311", 102.43e6),
 }
 
 # FFT kernels run out of shared memory and are limited by instruction issue,

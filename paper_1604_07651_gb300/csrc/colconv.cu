@@ -34,8 +34,8 @@ namespace hr {
 // columns, of which shared memory holds only one or two per SM.
 constexpr int kColThreads = 160;
 constexpr int kColThreadsMax = 384;
-// 480 threads at 128 registers fill the register file: three CTAs of 160, two
-// of 192 to 224, one of 256 and more.
+// Bounds a thread to 128 registers, so that the register file holds three CTAs
+// of 160 threads, two of 192 to 256, one of more.
 constexpr int kColThreadsReg = 480;
 // Twiddles of the middle passes (all but the first and the last), kept in
 // shared memory.

@@ -104,7 +104,7 @@ struct PieceDev {
 };
 
 // Up to kMaxBatch sub-problems launched as one grid: the blocks of piece k
-// are [first[k], first[k+1]); passed by value (about 3.3 KB of parameters).
+// are [first[k], first[k+1]); passed by value (about 4.7 KB of parameters).
 constexpr int kMaxBatch = 8;
 // Time pieces of one output column at most (RADON_MAX_TSPLIT + 1).
 constexpr int kMaxColPieces = 9;

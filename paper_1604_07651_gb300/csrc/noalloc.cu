@@ -26,7 +26,7 @@ static __device__ __align__(256) unsigned char g_noalloc_work[RADON_NOALLOC_MAX_
 
 namespace hr {
 
-// The piece descriptors of one call travel as a kernel parameter (about 13 KB
+// The piece descriptors of one call travel as a kernel parameter (about 19 KB
 // for 32 pieces, under the 32 KB parameter limit) and one small kernel writes
 // them into the work area: no host-to-device copy from pageable memory, which
 // would make the host wait for the stream.

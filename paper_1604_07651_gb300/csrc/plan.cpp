@@ -695,7 +695,8 @@ radon_status build_tile_lists(radon_plan_s* p, HostPiece& h, PieceDev& P) {
     // work units: every tile's chunks cut into pieces of at most kUnitChunks
     // chunks, each with the exponent of the largest B-spline weight sum a
     // cell of the tile collects from the unit's samples (the fixed-point
-    // bound of the kernel, computed with the kernel's own weights)
+    // bound of the kernel; its weights may differ from these in the last bits,
+    // far within the factor of two between the bound and a sum's range)
     std::vector<int4> flat, units;
     std::vector<long> uwork;
     std::vector<double> cell((size_t)TR * TC);
